@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
                  const T *__restrict__ base, const T *__restrict__ detail,
                  const T *__restrict__ weather, unsigned long long *__restrict__ counter) {
     __shared__ WarpScratch<CH, FX> scratch[4];
-    const unsigned long long n = march_tile<T, LS, SHAPE, FX, CH>(
+    const unsigned n = march_tile<T, LS, SHAPE, FX, CH>(
         p, v, blockIdx.x, blockIdx.y, scratch[threadIdx.x >> 5], base, detail, weather);
     count_lookups(counter, n);
 }
