@@ -96,7 +96,7 @@ int build_table(cloud_batch *b, cudaStream_t s) {
                                 cv.jitter_frame, cv.out_rgba, config_shape(b->config), &v))
             return rc;
         v.tile_begin = next;
-        next += v.tile_count;
+        next += tile_count(v, config_shape(b->config));
     }
     b->total_tiles = next;
     return check_cuda(cudaMemcpyAsync(b->d_views, b->table.data(), sizeof(ViewParams) * b->n_views,
@@ -305,7 +305,7 @@ extern "C" int cloud_batch_render_static(const cloud_volume *vol, const cloud_pa
                                 cv.out_rgba, config_shape(config), &table[q]))
             return rc;
         table[q].tile_begin = next;
-        next += table[q].tile_count;
+        next += tile_count(table[q], config_shape(config));
     }
     void *base = nullptr;
     if (int rc = static_scratch_address(&base)) return rc;

@@ -175,15 +175,25 @@ __device__ __forceinline__ df df_rsqrt(df a) {
 __device__ __forceinline__ bool df_gt(df a, df b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }
 __device__ __forceinline__ df df_max(df a, df b) { return df_gt(a, b) ? a : b; }
 __device__ __forceinline__ df df_min(df a, df b) { return df_gt(a, b) ? b : a; }
-// round(a) modulo 2^32 (fixed-point wrap) of a double-float with |a| < 2^55:
-// k = round(a.hi / 2^32) and r = a.hi - k 2^32 are exact (|r| <= 2^31, a
-// multiple of ulp(a.hi)); the integer part of r and the rounded remainder
-// (r - round(r)) + a.lo are converted with 32-bit conversions only.
-__device__ __forceinline__ uint32_t df_to_u32(df a) {
-    const float k = rintf(a.hi * 2.3283064365386963e-10f);
-    const float r = fmaf(-k, 4294967296.0f, a.hi);
-    const float rr = rintf(r);
-    return (uint32_t)__float2int_rn(rr) + (uint32_t)__float2int_rn((r - rr) + a.lo);
+// a b without the final renormalisation (|lo| up to a few ulp(hi)): four
+// operations, for a product that is only scaled again or rounded to fixed point.
+__device__ __forceinline__ df df_mul_raw(df a, df b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    const float e = fmaf(a.hi, b.hi, -p);
+    return {p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e))};
+}
+// round(a) modulo 2^32 (fixed-point wrap) of a double-float (lo up to a few
+// ulp(hi)) with |a| < 2^42, or < 2^54 if `wide`.  Additions only, no conversion
+// instruction (those run at a quarter of the rate or less): adding 1.5 2^43
+// leaves a.hi / 2^20, rounded, in the low mantissa bits (its low 12 bits are
+// the top 12 of the result); the exact remainder, below 2^19, plus a.lo is
+// rounded to an integer the same way.  `wide` first takes a multiple of 2^32
+// off a.hi, exactly.
+__device__ __forceinline__ uint32_t df_to_u32(df a, bool wide) {
+    if (wide) a.hi = fmaf(-rintf(a.hi * 2.3283064365386963e-10f), 4294967296.0f, a.hi);
+    const float t = __fadd_rn(a.hi, 0x1.8p43f);
+    const float s = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(t, 0x1.8p43f)), a.lo);
+    return (__float_as_uint(t) << 20) + (__float_as_uint(__fadd_rn(s, 0x1.8p23f)) - 0x4B400000u);
 }
 
 // Host: split an FP64 value into a double-float pair.

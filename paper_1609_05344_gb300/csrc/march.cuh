@@ -118,10 +118,10 @@ struct SceneParams {
     unsigned *check;  // status word of the checked build, else nullptr
     int log2_base, log2_detail, log2_weather;
     int light_steps, integration, constant_mode;
+    int wide;  // t_max spans more than 1000 tile periods (df_to_u32)
     // detail coordinates = (base + half_base) << detail_shift - half_detail when
     // the base tile period is 2^detail_shift detail periods (-1: convert separately)
     int detail_shift;
-    uint32_t jitter_key;
 };
 
 // One camera view: rays, layer clip, step count, jitter frame, output.
@@ -129,7 +129,8 @@ struct ViewParams {
     // Camera rays, unnormalised: v(x, y) = v00 + x vx + y vy, as double-float
     // pairs; vx/vy are split so that x * hi is exact (see split_df10).
     float v00h[3], v00l[3], vxh[3], vxl[3], vyh[3], vyl[3];
-    float oh[3], ol[3];    // camera position
+    uint32_t org[kLatticeAxes];  // camera position in fixed-point lattice coordinates, half_unit taken off
+    uint32_t org_h;              // camera height above the layer bottom in 2^-16 m
     float zlo_h, zlo_l;    // slab_lo - o_z
     float zhi_h, zhi_l;    // slab_hi - o_z
     float tmax_h, tmax_l;  // far clip distance
@@ -137,11 +138,11 @@ struct ViewParams {
     // rays with d_z below miss_below (camera under the layer) or above
     // miss_above (camera over it) cannot reach the layer within t_max
     float miss_below, miss_above;
-    int cam_in_layer, width, height, steps, jitter_frame;
-    float u_frame;   // >= 0: the start offset of every ray (per-frame jitter); < 0: per pixel
-    int tiles_x;     // tiles per image row
-    int tile_begin;  // first work-queue index of this view (multi-view launches)
-    int tile_count;
+    int width, height, steps;
+    float u_frame;         // >= 0: the start offset of every ray (no or per-frame jitter); < 0: per pixel
+    uint32_t jitter_hash;  // the part of the per-pixel hash that the frame and the seed decide
+    int tiles_x;           // tiles per image row
+    int tile_begin;        // first work-queue index of this view (multi-view launches)
     float4 *out;     // device RGBA, width * height
 };
 
@@ -418,32 +419,35 @@ __device__ __forceinline__ unsigned march_tile(
         };
         df lam0 = {0.0f, 0.0f}, lam1;
         if (fabsf(r[2].hi) * rnf < 1e-8f) {
-            alive = v.cam_in_layer != 0;
+            alive = v.zlo_h <= 0.0f && v.zhi_h >= 0.0f;  // the camera is in the layer
             lam1 = lam_max();
         } else {
+            // the sign of the ray's z decides which layer boundary comes first
             const df inv = df_recip(r[2]);
-            const df ll = df_mul({v.zlo_h, v.zlo_l}, inv), lh = df_mul({v.zhi_h, v.zhi_l}, inv);
-            lam0 = df_max(df_min(ll, lh), lam0);
-            lam1 = df_max(ll, lh);
+            const bool up = r[2].hi > 0.0f;
+            lam0 = df_mul({up ? v.zlo_h : v.zhi_h, up ? v.zlo_l : v.zhi_l}, inv);
+            lam1 = df_mul({up ? v.zhi_h : v.zlo_h, up ? v.zhi_l : v.zlo_l}, inv);
+            if (!(lam0.hi > 0.0f)) lam0 = {0.0f, 0.0f};
             if (!(lam1.hi < v.tmax_h * rnf * (1.0f - 1e-5f))) lam1 = df_min(lam1, lam_max());
             alive = df_gt(lam1, lam0);
         }
         if (alive) {
             // --- a2: jittered start offset (Sec. 3.2) ---------------------------
             const df D = df_mul(df_add(lam1, df_neg(lam0)), {v.invn_h, v.invn_l});
-            float u = 0.5f;
-            if (v.u_frame >= 0.0f)
-                u = v.u_frame;
-            else if (v.jitter_frame >= 0)
-                u = (float)(pcg_hash4((uint32_t)x, (uint32_t)y, (uint32_t)v.jitter_frame,
-                                      p.jitter_key) >> 8) * (1.0f / 16777216.0f);
+            float u = v.u_frame;
+            if (u < 0.0f)
+                u = (float)(pcg_hash((uint32_t)x ^ pcg_hash((uint32_t)y ^ v.jitter_hash)) >> 8) *
+                    (1.0f / 16777216.0f);
             const df lam_s = df_add(lam0, df_mulf(D, u));
+            // start and step of every axis: (lambda v) scaled to the axis' units and
+            // rounded to fixed point, the camera's own coordinate added as an integer
             df pos[3], dpos[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                pos[k] = df_add({v.oh[k], v.ol[k]}, df_mul(lam_s, r[k]));
-                dpos[k] = df_mul(D, r[k]);
+                pos[k] = df_mul_raw(lam_s, r[k]);
+                dpos[k] = df_mul_raw(D, r[k]);
             }
+            const bool wide = p.wide != 0;
 #pragma unroll
             for (int a = 0; a < kLatticeAxes; ++a) {
                 const int comp = a < 6 ? a % 3 : a - 6;
@@ -455,13 +459,12 @@ __device__ __forceinline__ unsigned march_tile(
                     continue;
                 }
                 const df k = {p.kfix_h[a], p.kfix_l[a]};
-                c[a] = df_to_u32(df_mul(pos[comp], k)) - p.half_unit[a];
-                e[a] = df_to_u32(df_mul(dpos[comp], k));
+                c[a] = df_to_u32(df_mul_raw(pos[comp], k), wide) + v.org[a];
+                e[a] = df_to_u32(df_mul_raw(dpos[comp], k), wide);
             }
-            // height above the layer bottom: (o_z - slab_lo) + lambda v_z, in 2^-16 m
-            const df hrel = df_add(df_mul(lam_s, r[2]), df_neg({v.zlo_h, v.zlo_l}));
-            hq = (int32_t)df_to_u32({hrel.hi * 65536.0f, hrel.lo * 65536.0f});
-            eh = (int32_t)df_to_u32({dpos[2].hi * 65536.0f, dpos[2].lo * 65536.0f});
+            // height above the layer bottom, in 2^-16 m
+            hq = (int32_t)(df_to_u32({pos[2].hi * 65536.0f, pos[2].lo * 65536.0f}, false) + v.org_h);
+            eh = (int32_t)df_to_u32({dpos[2].hi * 65536.0f, dpos[2].lo * 65536.0f}, false);
             const float vlen = n2f * rnf;
             Df = D.hi * vlen;
             // --- a5: phase function, hoisted per ray ----------------------------
@@ -640,6 +643,12 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
                 SceneParams *p);
 int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_camera *cam, int width,
                int height, int steps, int jitter_frame, float *out, int shape, ViewParams *v);
+// Pixel tiles of a view in a launch of the given tile shape.
+inline int tile_count(const ViewParams &v, int shape) {
+    int tw, th;
+    tile_dims(shape, &tw, &th);
+    return v.tiles_x * ((v.height + th - 1) / th);
+}
 // The autotuned launch configuration for (storage precision, light steps).
 int tuned_config(int precision, int light_steps);
 // Raymarch of one view with the given configuration (render.cu); the

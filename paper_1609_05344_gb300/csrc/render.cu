@@ -6,6 +6,7 @@
 // touch the same region of the L2-resident noise tiles.  The device code is
 // in march.cuh, the kernels in march_kernels.cuh (instantiated by
 // march{8,16}_{view,batch}.cu).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <mutex>
@@ -92,13 +93,16 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
     p->light_steps = light_steps;
     p->integration = integration;
     p->constant_mode = noise ? 0 : 1;
+    double least_period = d.base_period_m;
+    if (noise && vol->log2_detail) least_period = std::min(least_period, d.detail_period_m);
+    if (noise && vol->log2_weather) least_period = std::min(least_period, d.weather_period_m);
+    p->wide = noise && !(prm->t_max_m < 1000.0 * least_period);
     p->detail_shift = -1;
     if (vol->log2_detail) {
         const double ratio = d.base_period_m / d.detail_period_m;
         for (int k = 0; k <= 16; ++k)
             if (ratio == std::ldexp(1.0, k)) p->detail_shift = k;
     }
-    p->jitter_key = d.seed ^ kJitterKey;
     return CLOUD_OK;
 }
 
@@ -121,13 +125,26 @@ int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_cam
         split_df(cam->forward[k] + a0 * cam->right[k] + b0 * cam->up[k], &v->v00h[k], &v->v00l[k]);
         split_df10(ax * cam->right[k], &v->vxh[k], &v->vxl[k]);
         split_df10(by * cam->up[k], &v->vyh[k], &v->vyl[k]);
-        split_df(cam->pos[k], &v->oh[k], &v->ol[k]);
     }
+    if (d.density_mode == CLOUD_DENSITY_NOISE) {
+        const double P[kLatticeAxes] = {d.base_period_m,    d.base_period_m,    d.base_period_m,
+                                        d.detail_period_m,  d.detail_period_m,  d.detail_period_m,
+                                        d.weather_period_m, d.weather_period_m};
+        const int L[kLatticeAxes] = {vol->log2_base,    vol->log2_base,    vol->log2_base,
+                                     vol->log2_detail,  vol->log2_detail,  vol->log2_detail,
+                                     vol->log2_weather, vol->log2_weather};
+        for (int a = 0; a < kLatticeAxes; ++a) {
+            if (L[a] == 0) continue;  // absent tile: axis unused
+            const double t = cam->pos[a < 6 ? a % 3 : a - 6] / P[a];
+            v->org[a] = (uint32_t)(unsigned long long)std::llrint((t - std::floor(t)) * 4294967296.0) -
+                        (1u << (31 - L[a]));
+        }
+    }
+    v->org_h = (uint32_t)(unsigned long long)std::llrint((cam->pos[2] - d.slab_lo_m) * 65536.0);
     split_df(d.slab_lo_m - cam->pos[2], &v->zlo_h, &v->zlo_l);
     split_df(d.slab_hi_m - cam->pos[2], &v->zhi_h, &v->zhi_l);
     split_df(prm->t_max_m, &v->tmax_h, &v->tmax_l);
     split_df(1.0 / steps, &v->invn_h, &v->invn_l);
-    v->cam_in_layer = cam->pos[2] >= d.slab_lo_m && cam->pos[2] <= d.slab_hi_m;
     // a ray from below reaches the layer within t_max only if d_z >= (lo - o_z)/t_max
     v->miss_below = -INFINITY;
     v->miss_above = INFINITY;
@@ -138,15 +155,17 @@ int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_cam
     v->width = width;
     v->height = height;
     v->steps = steps;
-    v->jitter_frame = jitter_frame < 0 ? -1 : jitter_frame;
-    v->u_frame = -1.0f;
-    if (jitter_frame >= 0 && prm->jitter_mode == CLOUD_JITTER_PER_FRAME)  // offset of pixel (0, 0)
-        v->u_frame = (float)(pcg_hash4(0u, 0u, (uint32_t)jitter_frame, d.seed ^ kJitterKey) >> 8) *
-                     (1.0f / 16777216.0f);
+    v->u_frame = 0.5f;
+    if (jitter_frame >= 0) {
+        v->jitter_hash = pcg_hash((uint32_t)jitter_frame ^ pcg_hash(d.seed ^ kJitterKey));
+        v->u_frame = -1.0f;
+        if (prm->jitter_mode == CLOUD_JITTER_PER_FRAME)  // offset of pixel (0, 0)
+            v->u_frame = (float)(pcg_hash4(0u, 0u, (uint32_t)jitter_frame, d.seed ^ kJitterKey) >> 8) *
+                         (1.0f / 16777216.0f);
+    }
     int tw, th;
     tile_dims(shape, &tw, &th);
     v->tiles_x = (width + tw - 1) / tw;
-    v->tile_count = v->tiles_x * ((height + th - 1) / th);
     v->out = (float4 *)out;
     return CLOUD_OK;
 }

@@ -166,7 +166,7 @@ int launch_slot(cloud_server *srv, int si, const std::vector<Request *> &batch) 
                                 se.current, config_shape(srv->config), &v))
             return rc;
         v.tile_begin = next;
-        next += v.tile_count;
+        next += tile_count(v, config_shape(srv->config));
     }
     if (int rc = check_cuda(cudaMemcpyAsync(sl.d_table, sl.h_table, sizeof(ViewParams) * n,
                                             cudaMemcpyHostToDevice, sl.stream),
