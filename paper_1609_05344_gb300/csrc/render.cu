@@ -103,6 +103,15 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
         for (int k = 0; k <= 16; ++k)
             if (ratio == std::ldexp(1.0, k)) p->detail_shift = k;
     }
+    if (p->detail_shift >= 0) {
+        p->detail_mul = 1u << p->detail_shift;
+        p->detail_add = (p->half_unit[kBX] << p->detail_shift) - p->half_unit[kDX];
+    }
+    p->base_mul[0] = 1u << vol->log2_base;
+    p->base_mul[1] = 1u << (2 * vol->log2_base);
+    p->detail_rec_mul[0] = 1u << vol->log2_detail;
+    p->detail_rec_mul[1] = 1u << (2 * vol->log2_detail);
+    p->weather_mul = 1u << vol->log2_weather;
     return CLOUD_OK;
 }
 

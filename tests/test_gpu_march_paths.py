@@ -1,0 +1,72 @@
+"""GPU parity of the raymarch's special paths against the FP64 oracle: tile
+periods so short that a ray spans thousands of them, light samples that leave
+the layer, step counts that do not fill a chunk, and rays in clear air.
+
+Tolerances (max-abs RGBA) are those of every other render: 1e-4 for FP32
+volumes, 3e-3 for FP16 volumes."""
+import numpy as np
+import pytest
+
+from paper_1609_05344_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp32": 1e-4, "fp16": 3e-3}
+
+
+@pytest.fixture(scope="module")
+def api():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1609_05344_gb300 import _native, api as A
+    _native.build()
+    return A
+
+
+def _check(api, oracle, desc, prm, cam, w, h, steps, light_steps, frame=-1):
+    vol, ovol = api.Volume(desc), oracle.Volume(desc)
+    got, count = api.render(vol, cam, prm, w, h, steps, light_steps, jitter_frame=frame, count=True)
+    ref, n = oracle.render(ovol, cam, prm, w, h, steps, light_steps, jitter_frame=frame, nthreads=8)
+    assert np.abs(got.cpu().numpy() - ref).max() <= TOL[desc["precision"]]
+    return ref, int(count.item()), n
+
+
+# 40 km rays: 1000 periods of 39 m or less take the reduction modulo 2^32
+@pytest.mark.parametrize("kind,base_period", [("tiny", 39.0), ("tiny", 41.0), ("full", 256.0),
+                                              ("full", 400.0)])
+@pytest.mark.parametrize("height", [500.0, 2500.0])
+def test_short_tile_periods(api, oracle, kind, base_period, height):
+    desc = I.volume_desc(kind, seed=5, base_period=base_period, detail_period=base_period / 8.0)
+    cam = I.camera((12345.6, -2345.6, height), 33.0, 36.0, 60.0)
+    ref, _, _ = _check(api, oracle, desc, I.params(), cam, 45, 31, 9, 6, frame=2)
+    assert ref[..., 3].max() > 0.1
+
+
+# the light march ends 2.0 km (0.8 km, 0.5 km) above its view sample in a 2.5 km layer
+@pytest.mark.parametrize("light_step,light_steps", [(420.0, 6), (180.0, 6), (100.0, 9)])
+@pytest.mark.parametrize("kind,precision", [("full", "fp32"), ("full", "fp16"), ("tiny", "fp32")])
+@pytest.mark.parametrize("height,pitch", [(500.0, 36.0), (5200.0, -40.0)])
+def test_light_samples_above_the_layer(api, oracle, light_step, light_steps, kind, precision, height,
+                                       pitch):
+    desc = I.volume_desc(kind, seed=6, precision=precision)
+    cam = I.camera((800.0, 300.0, height), 120.0, pitch, 60.0)
+    ref, _, _ = _check(api, oracle, desc, I.params(light_step=light_step), cam, 40, 27, 17,
+                       light_steps, frame=3)
+    assert ref[..., 3].max() > 0.1
+
+
+# 1 and 7: part of a chunk; 11 and 17: whole chunks and a part; 130: mostly clear chunks
+@pytest.mark.parametrize("steps", [1, 7, 11, 17, 130])
+@pytest.mark.parametrize("config", [0, 4])
+def test_partial_and_clear_chunks(api, oracle, steps, config):
+    desc = I.volume_desc("full", seed=7)
+    api.set_launch_config("fp32", 6, config)
+    try:
+        cam = I.camera((0.0, 0.0, 500.0), 70.0, 36.0, 60.0)
+        ref, count, n = _check(api, oracle, desc, I.params(), cam, 33, 18, steps, 6)
+    finally:
+        api.set_launch_config("fp32", 6, 3)
+    # lookups in the method's sense: a density within rounding of 0, or an optical depth
+    # within rounding of the early out, may move single steps of single rays
+    assert abs(count - n) <= 1e-3 * n + 6
