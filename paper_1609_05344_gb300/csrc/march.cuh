@@ -214,8 +214,12 @@ struct WarpScratch {
     uint16_t pairs[CH * 32];
 };
 
-__device__ __forceinline__ float frac23(uint32_t f) {
-    return __uint_as_float((f >> 9) | 0x3F800000u) - 1.0f;
+// Two interpolation weights (23 bits below the index bits, shifted to the top)
+// with one packed subtraction.
+__device__ __forceinline__ float2 frac23(uint32_t f, uint32_t g) {
+    return __fadd2_rn(make_float2(__uint_as_float((f >> 9) | 0x3F800000u),
+                                  __uint_as_float((g >> 9) | 0x3F800000u)),
+                      make_float2(-1.0f, -1.0f));
 }
 
 // a b + c (mod 2^32) as one integer multiply-add, whatever b is.
@@ -239,9 +243,7 @@ __device__ __forceinline__ uint32_t rec2(uint32_t mul, int L, uint32_t cx, uint3
 // (z0, z1) pairs of both y rows (the x differences come with the record),
 // then y on the pair, then z.  Each lane of a packed op rounds exactly like
 // the scalar op.
-__device__ __forceinline__ float trilerp(const float c[8], int L, uint32_t cx, uint32_t cy,
-                                         uint32_t cz) {
-    const float fx = frac23(cx << L), fy = frac23(cy << L), fz = frac23(cz << L);
+__device__ __forceinline__ float trilerp(const float c[8], float fx, float fy, float fz) {
     const float2 a0 = make_float2(c[0], c[1]), a1 = make_float2(c[2], c[3]);  // dx = 0
     const float2 d0 = make_float2(c[4], c[5]), d1 = make_float2(c[6], c[7]);  // dx = 1 minus dx = 0
     const float2 fx2 = make_float2(fx, fx), fy2 = make_float2(fy, fy);
@@ -250,8 +252,7 @@ __device__ __forceinline__ float trilerp(const float c[8], int L, uint32_t cx, u
     const float2 yz = __ffma2_rn(fy2, __fadd2_rn(x1, make_float2(-x0.x, -x0.y)), x0);  // (z0, z1)
     return fmaf(fz, yz.y - yz.x, yz.x);
 }
-__device__ __forceinline__ float bilerp(const float c[4], int L, uint32_t cx, uint32_t cy) {
-    const float fx = frac23(cx << L), fy = frac23(cy << L);
+__device__ __forceinline__ float bilerp(const float c[4], float fx, float fy) {
     const float2 a = make_float2(c[0], c[1]), d = make_float2(c[2], c[3]);  // (y0, y1): dx = 0, difference
     const float2 xy = __ffma2_rn(make_float2(fx, fx), d, a);
     return fmaf(fy, xy.y - xy.x, xy.x);
@@ -319,14 +320,16 @@ __device__ __forceinline__ Density density(const SceneParams &p, const T *__rest
     float od = 0.0f, ow = 0.0f;
     if (FX || detail) od = load_rec8(detail, rd, cd);
     if (FX || weather) ow = load_rec4(weather, rw, cw);
-    const float b = trilerp(cb, lb, c[kBX], c[kBY], c[kBZ]) + ob;
+    const float2 fb = frac23(c[kBX] << lb, c[kBY] << lb), fd = frac23(c[kDX] << ld, c[kDY] << ld),
+                 fz = frac23(c[kBZ] << lb, c[kDZ] << ld), fw = frac23(c[kWX] << lw, c[kWY] << lw);
+    const float b = trilerp(cb, fb.x, fb.y, fz.x) + ob;
     float r = b + p.k0;
     if (FX || detail) {
-        const float dt = trilerp(cd, ld, c[kDX], c[kDY], c[kDZ]) + od;
+        const float dt = trilerp(cd, fd.x, fd.y, fz.y) + od;
         r = fmaf(-p.detail_w, dt, r);
     }
     r = fmaxf(r * p.inv_1mc, 0.0f);
-    const float w = (FX || weather) ? bilerp(cw, lw, c[kWX], c[kWY]) + ow + p.w_off : 1.0f;
+    const float w = (FX || weather) ? bilerp(cw, fw.x, fw.y) + ow + p.w_off : 1.0f;
     return {__fmul_rn(g, w), r};
 }
 
@@ -521,33 +524,38 @@ __device__ __forceinline__ unsigned march_tile(
         const int nst = min(CH, v.steps - i0);
         // --- A1: which of this lane's CH steps need a density lookup: those in an
         //     occupied macro-cell of the occupancy grid (the grid words of all CH
-        //     steps are loaded together).  A step outside the layer, possible only
-        //     by rounding at the ends of the clipped ray, is left to the lookup. ---
-        uint32_t need = 0;
-        if (alive) {
-            if ((FX || !p.constant_mode) && p.occ) {
-                const uint4 s = ws.ray[lane][0], d = ws.ray[lane][1];
-                uint32_t bx = s.x + i0 * d.x, by = s.y + i0 * d.y, bz = s.z + i0 * d.z;
+        //     steps are loaded together, by every lane: the coordinates of a
+        //     finished ray and of steps past the last wrap into the grid too).  A
+        //     step outside the layer, possible only by rounding at the ends of the
+        //     clipped ray, is left to the lookup. -------------------------------
+        bool occ[CH];
+        if ((FX || !p.constant_mode) && p.occ) {
+            const uint4 s = ws.ray[lane][0], d = ws.ray[lane][1];
+            uint32_t bx = s.x + i0 * d.x, by = s.y + i0 * d.y, bz = s.z + i0 * d.z;
 #pragma unroll
-                for (int k = 0; k < CH; ++k) {
-                    if (k < nst && occupied<FX>(p, bx, by, bz)) need |= 1u << k;
-                    bx += d.x;
-                    by += d.y;
-                    bz += d.z;
-                }
-            } else {
-                need = (1u << nst) - 1u;
+            for (int k = 0; k < CH; ++k) {
+                occ[k] = occupied<FX>(p, bx, by, bz);
+                bx += d.x;
+                by += d.y;
+                bz += d.z;
             }
+        } else {
+#pragma unroll
+            for (int k = 0; k < CH; ++k) occ[k] = true;
         }
         // --- A2: those (step, lane) lookups shared out over the warp, one or two
         //     per lane at a time (ViewBatch) so that their loads overlap (a3) ---
+        uint32_t need = 0;
         unsigned nq = 0;
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
-            const unsigned m = __ballot_sync(kFull, (need >> k) & 1u);
+            const bool nd = occ[k] && alive && k < nst;
+            const unsigned m = __ballot_sync(kFull, nd);
             const unsigned slot = nq + __popc(m & lt_mask);
-            if (((need >> k) & 1u) && in_range(p.check, slot < CH * 32u, kChkWork))
-                ws.pairs[slot] = (uint16_t)((k << 5) | lane);
+            if (nd) {
+                need |= 1u << k;
+                if (in_range(p.check, slot < CH * 32u, kChkWork)) ws.pairs[slot] = (uint16_t)((k << 5) | lane);
+            }
             nq += __popc(m);
         }
         if (nq == 0) {  // clear air, warp-wide: no optical depth, no early out
