@@ -156,11 +156,18 @@ __device__ __forceinline__ df df_mulf(df a, float b) {
     const float e = fmaf(a.hi, b, -p);
     return fast_two_sum(p, fmaf(a.lo, b, e));
 }
-// 1/b: one Newton step on the hardware reciprocal estimate (PTX rcp.approx,
-// relative error about 2^-23; the step squares it, like df_rsqrt's).
+// Reciprocal square root of a normal number (rsqrtf without its scaling of
+// subnormal arguments; the same value).
+__device__ __forceinline__ float rsqrt_norm(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// 1/b of a normal b: one Newton step on the hardware reciprocal estimate (PTX
+// rcp.approx, relative error about 2^-23; the step squares it, like df_rsqrt's).
 __device__ __forceinline__ df df_recip(df b) {
     float q;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(q) : "f"(b.hi));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(b.hi));
     const df p = df_mulf(b, q);                 // b q = 1 - r
     const float r = (1.0f - p.hi) - p.lo;
     return fast_two_sum(q, q * r);

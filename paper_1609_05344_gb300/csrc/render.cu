@@ -112,6 +112,7 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
     p->detail_rec_mul[0] = 1u << vol->log2_detail;
     p->detail_rec_mul[1] = 1u << (2 * vol->log2_detail);
     p->weather_mul = 1u << vol->log2_weather;
+    p->one = 1u;
     return CLOUD_OK;
 }
 
