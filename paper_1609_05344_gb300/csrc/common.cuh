@@ -182,25 +182,49 @@ __device__ __forceinline__ df df_rsqrt(df a) {
 __device__ __forceinline__ bool df_gt(df a, df b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }
 __device__ __forceinline__ df df_max(df a, df b) { return df_gt(a, b) ? a : b; }
 __device__ __forceinline__ df df_min(df a, df b) { return df_gt(a, b) ? b : a; }
-// a b without the final renormalisation (|lo| up to a few ulp(hi)): four
-// operations, for a product that is only scaled again or rounded to fixed point.
-__device__ __forceinline__ df df_mul_raw(df a, df b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    const float e = fmaf(a.hi, b.hi, -p);
-    return {p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e))};
+// Two double-floats side by side, on Blackwell's packed FP32x2 operations: one
+// instruction a pair, each lane rounded like the scalar one.
+struct df2 {
+    float2 hi, lo;
+};
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ df2 fast_two_sum2(float2 a, float2 b) {  // requires |a| >= |b|
+    const float2 s = __fadd2_rn(a, b);
+    return {s, sub2(b, sub2(s, a))};
 }
-// round(a) modulo 2^32 (fixed-point wrap) of a double-float (lo up to a few
-// ulp(hi)) with |a| < 2^42, or < 2^54 if `wide`.  Additions only, no conversion
-// instruction (those run at a quarter of the rate or less): adding 1.5 2^43
-// leaves a.hi / 2^20, rounded, in the low mantissa bits (its low 12 bits are
-// the top 12 of the result); the exact remainder, below 2^19, plus a.lo is
+__device__ __forceinline__ df2 two_sum2(float2 a, float2 b) {
+    const float2 s = __fadd2_rn(a, b);
+    const float2 bb = sub2(s, a);
+    return {s, __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+// a b without the final renormalisation (|lo| up to a few ulp(hi)), for a product
+// that is only scaled again or rounded to fixed point.
+__device__ __forceinline__ df2 df2_mul_raw(df2 a, df2 b) {
+    const float2 p = __fmul2_rn(a.hi, b.hi);
+    const float2 e = __ffma2_rn(a.hi, b.hi, neg2(p));
+    return {p, __ffma2_rn(a.hi, b.lo, __ffma2_rn(a.lo, b.hi, e))};
+}
+// round(a) modulo 2^32 (fixed-point wrap) of each of two double-floats (lo up to
+// a few ulp(hi)) with |a| < 2^42, or < 2^54 if `wide`.  Additions only, no
+// conversion instruction (those run at a quarter of the rate or less): adding
+// 1.5 2^43 leaves a.hi / 2^20, rounded, in the low mantissa bits (its low 12 bits
+// are the top 12 of the result); the exact remainder, below 2^19, plus a.lo is
 // rounded to an integer the same way.  `wide` first takes a multiple of 2^32
-// off a.hi, exactly.
-__device__ __forceinline__ uint32_t df_to_u32(df a, bool wide) {
-    if (wide) a.hi = fmaf(-rintf(a.hi * 2.3283064365386963e-10f), 4294967296.0f, a.hi);
-    const float t = __fadd_rn(a.hi, 0x1.8p43f);
-    const float s = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(t, 0x1.8p43f)), a.lo);
-    return (__float_as_uint(t) << 20) + (__float_as_uint(__fadd_rn(s, 0x1.8p23f)) - 0x4B400000u);
+// off a.hi, exactly, and renormalises (lo may be far above 2^22 there).
+__device__ __forceinline__ uint2 df2_to_u32(df2 a, bool wide) {
+    if (wide) {
+        a.hi = __ffma2_rn(make_float2(-rintf(a.hi.x * 2.3283064365386963e-10f),
+                                      -rintf(a.hi.y * 2.3283064365386963e-10f)),
+                          both(4294967296.0f), a.hi);
+        a = two_sum2(a.hi, a.lo);
+    }
+    const float2 t = __fadd2_rn(a.hi, both(0x1.8p43f));
+    const float2 s = __fadd2_rn(sub2(a.hi, __fadd2_rn(t, both(-0x1.8p43f))), a.lo);
+    const float2 u = __fadd2_rn(s, both(0x1.8p23f));
+    return make_uint2((__float_as_uint(t.x) << 20) + (__float_as_uint(u.x) - 0x4B400000u),
+                      (__float_as_uint(t.y) << 20) + (__float_as_uint(u.y) - 0x4B400000u));
 }
 
 // Host: split an FP64 value into a double-float pair.

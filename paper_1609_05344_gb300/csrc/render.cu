@@ -55,7 +55,9 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
         const int comp = a < 6 ? a % 3 : a - 6;
         if (!noise || L[a] == 0) continue;  // absent tile: axis unused
         const double kfix = 4294967296.0 / P[a];  // 2^32 fixed-point units per tile
-        split_df(kfix, &p->kfix_h[a], &p->kfix_l[a]);
+        split_df(kfix, &p->kfix_h[a].x, &p->kfix_l[a].x);
+        p->kfix_h[a].y = p->kfix_h[a].x;
+        p->kfix_l[a].y = p->kfix_l[a].x;
         p->half_unit[a] = 1u << (31 - L[a]);
         for (int j = 0; j < light_steps; ++j) {
             const double off = (j + 0.5) * prm->light_step_m * s[comp] * kfix;

@@ -32,8 +32,10 @@ def _check(api, oracle, desc, prm, cam, w, h, steps, light_steps, frame=-1):
     return ref, int(count.item()), n
 
 
-# 40 km rays: 1000 periods of 39 m or less take the reduction modulo 2^32
-@pytest.mark.parametrize("kind,base_period", [("tiny", 39.0), ("tiny", 41.0), ("full", 256.0),
+# 40 km rays: 1000 periods of 39 m or less take the reduction modulo 2^32; at 1 m a ray spans
+# 2^47 fixed-point units and the low part of the double-float product is far above one of them
+@pytest.mark.parametrize("kind,base_period", [("tiny", 1.0), ("tiny", 4.0), ("tiny", 39.0),
+                                              ("tiny", 41.0), ("full", 16.0), ("full", 256.0),
                                               ("full", 400.0)])
 @pytest.mark.parametrize("height", [500.0, 2500.0])
 def test_short_tile_periods(api, oracle, kind, base_period, height):
