@@ -163,11 +163,16 @@ __device__ __forceinline__ float rsqrt_norm(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// Reciprocal estimate of a normal number (PTX rcp.approx).
+__device__ __forceinline__ float rcp_norm(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 // 1/b of a normal b: one Newton step on the hardware reciprocal estimate (PTX
 // rcp.approx, relative error about 2^-23; the step squares it, like df_rsqrt's).
 __device__ __forceinline__ df df_recip(df b) {
-    float q;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(b.hi));
+    const float q = rcp_norm(b.hi);
     const df p = df_mulf(b, q);                 // b q = 1 - r
     const float r = (1.0f - p.hi) - p.lo;
     return fast_two_sum(q, q * r);

@@ -1,11 +1,11 @@
 // taa.cu -- reprojection motion and the temporal anti-aliasing resolve
 // (Sec. 3.2: jittered frames are accumulated by Playdead-style TAA).
 //
-// Both kernels are memory-bound streaming passes: one thread per pixel,
-// 32x8 CTAs, 16-byte RGBA loads/stores (8-byte for FP16 history).  The 3x3
-// neighbourhood reads of the current frame and the 2x2 history footprint are
-// served by L1; each pixel's own current value, motion and output are the
-// compulsory traffic.
+// Streaming passes over 32-pixel-wide tiles of 32x8 threads, several vertically
+// adjacent pixels a thread, 16-byte RGBA loads/stores (8-byte for FP16 history).
+// The current frame's 3x3 neighbourhoods come from a shared-memory tile, the 2x2
+// history footprint through L1; each pixel's own current value, history, motion
+// and output are the compulsory traffic.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -68,6 +68,9 @@ __device__ __noinline__ float entry_lambda_exact(const MotionParams &p, int x, i
 // parameter of the layer entry (FP32, with a flag for the near ties that the
 // double-float restatement decides), and the projection into the previous
 // camera.
+//
+// Two rows of a column at a time, on packed FP32x2 operations (the arithmetic is
+// what bounds the motion: 118 instructions a pixel one at a time).
 struct MotionCol {
     float a, n2x, vzx, gx0, gx1, gx2, akx, nx0;
 };
@@ -83,57 +86,94 @@ __device__ __forceinline__ MotionCol motion_col(const MotionParams &p, int x) {
     c.nx0 = fmaf(c.akx, p.dlt[2], -p.dlt[0]);
     return c;
 }
+// Slopes of rows y and y + 1.
+__device__ __forceinline__ float2 motion_rows(const MotionParams &p, int y) {
+    return make_float2(fmaf((float)y, p.by, p.b0), fmaf((float)(y + 1), p.by, p.b0));
+}
 // Depth parameter lambda (t / |v|) of the layer entry, or of the far clip;
 // *exact is set when FP32 cannot call the entry (the caller then takes
-// entry_lambda_exact).  b is the row slope.
-__device__ __forceinline__ float motion_lambda(const MotionParams &p, const MotionCol &c, float b,
-                                               bool *exact) {
-    const float n2 = fmaf(b, b, c.n2x);
-    const float vz = fmaf(b, p.uz, c.vzx);
+// entry_lambda_exact).
+__device__ __forceinline__ float motion_entry(const MotionParams &p, float lmax, float ll, float lh,
+                                              bool horizontal, bool *exact) {
+    const float l0 = fmaxf(fminf(ll, lh), 0.0f), l1 = fminf(fmaxf(ll, lh), lmax);
+    *exact = !horizontal && fabsf(l1 - l0) <= 1e-5f * fmaxf(l1, l0);  // too close to call in FP32
+    return !horizontal && l1 > l0 && l0 > 0.0f ? l0 : lmax;
+}
+// Both rows' lambda; b: the rows' slopes.
+__device__ __forceinline__ float2 motion_lambda(const MotionParams &p, const MotionCol &c, float2 b,
+                                                bool *exact0, bool *exact1) {
+    const float2 n2 = __ffma2_rn(b, b, both(c.n2x));
+    const float2 vz = __ffma2_rn(b, both(p.uz), both(c.vzx));
     // divisions by hardware reciprocals (relative error ~1e-7, far below the
-    // 1e-5 margin of the near-tie test and the motion's own accuracy)
-    const float lmax = p.tmax * rsqrtf(n2);
-    float lam = lmax;
-    *exact = false;
-    if (vz * vz >= 1e-16f * n2) {  // |d_z| >= 1e-8
-        const float ivz = __fdividef(1.0f, vz);
-        const float ll = p.zlo * ivz, lh = p.zhi * ivz;
-        const float l0 = fmaxf(fminf(ll, lh), 0.0f), l1 = fminf(fmaxf(ll, lh), lmax);
-        if (fabsf(l1 - l0) <= 1e-5f * fmaxf(l1, l0))
-            *exact = true;  // too close to call in FP32
-        else if (l1 > l0 && l0 > 0.0f)
-            lam = l0;
-    }
-    return lam;
+    // 1e-5 margin of the near-tie test and the motion's own accuracy) of normal
+    // numbers, without the scaling of subnormal ones
+    const float2 lmax = __fmul2_rn(both(p.tmax), make_float2(rsqrt_norm(n2.x), rsqrt_norm(n2.y)));
+    const float2 vz2 = __fmul2_rn(vz, vz), lim = __fmul2_rn(n2, both(1e-16f));
+    const float2 ivz = make_float2(rcp_norm(vz.x), rcp_norm(vz.y));
+    const float2 ll = __fmul2_rn(both(p.zlo), ivz), lh = __fmul2_rn(both(p.zhi), ivz);
+    // horizontal: |d_z| < 1e-8
+    return make_float2(motion_entry(p, lmax.x, ll.x, lh.x, !(vz2.x >= lim.x), exact0),
+                       motion_entry(p, lmax.y, ll.y, lh.y, !(vz2.y >= lim.y), exact1));
 }
-__device__ __forceinline__ float2 motion_project(const MotionParams &p, const MotionCol &c, float b,
-                                                 float lam) {
-    const float g0 = fmaf(p.G[0][1], b, c.gx0);
-    const float g1 = fmaf(p.G[1][1], b, c.gx1);
-    const float g2 = fmaf(p.G[2][1], b, c.gx2);
-    const float qz = fmaf(lam, 1.0f + g2, p.dlt[2]);
-    if (qz <= 0.0f) return make_float2(1e9f, 1e9f);
+// Both rows' motion: (x, y) of row y, then of row y + 1.
+__device__ __forceinline__ float4 motion_project(const MotionParams &p, const MotionCol &c, float2 b,
+                                                 float2 lam) {
+    const float2 g0 = __ffma2_rn(both(p.G[0][1]), b, both(c.gx0));
+    const float2 g1 = __ffma2_rn(both(p.G[1][1]), b, both(c.gx1));
+    const float2 g2 = __ffma2_rn(both(p.G[2][1]), b, both(c.gx2));
+    const float2 qz = __ffma2_rn(lam, __fadd2_rn(both(1.0f), g2), both(p.dlt[2]));
     // a kx qz - qx and qy - b ky qz, expanded so the O(lambda) terms cancel exactly
-    const float bky = b * p.ky;
-    const float nx = c.nx0 + lam * fmaf(c.a, p.kx1, fmaf(c.akx, g2, -g0));
-    const float ny = fmaf(-bky, p.dlt[2], p.dlt[1]) + lam * fmaf(-b, p.ky1, fmaf(-bky, g2, g1));
-    const float iq = __fdividef(1.0f, qz);
-    return make_float2(p.sx * nx * iq, p.sy * ny * iq);
+    const float2 nbky = __fmul2_rn(b, both(-p.ky));
+    const float2 nx = __ffma2_rn(lam, __ffma2_rn(both(c.a), both(p.kx1), __ffma2_rn(both(c.akx), g2, neg2(g0))),
+                                 both(c.nx0));
+    const float2 ny = __ffma2_rn(lam, __ffma2_rn(b, both(-p.ky1), __ffma2_rn(nbky, g2, g1)),
+                                 __ffma2_rn(nbky, both(p.dlt[2]), both(p.dlt[1])));
+    const float2 iq = make_float2(rcp_norm(qz.x), rcp_norm(qz.y));
+    const float2 mx = __fmul2_rn(__fmul2_rn(both(p.sx), nx), iq);
+    const float2 my = __fmul2_rn(__fmul2_rn(both(p.sy), ny), iq);
+    const bool on0 = qz.x > 0.0f, on1 = qz.y > 0.0f;  // not behind the previous camera
+    return make_float4(on0 ? mx.x : 1e9f, on0 ? my.x : 1e9f, on1 ? mx.y : 1e9f, on1 ? my.y : 1e9f);
 }
-__device__ __forceinline__ float2 motion_at(const MotionParams &p, int x, int y) {
-    const MotionCol c = motion_col(p, x);
-    const float b = fmaf((float)y, p.by, p.b0);
-    bool ex;
-    float lam = motion_lambda(p, c, b, &ex);
-    if (ex) lam = entry_lambda_exact(p, x, y);
-    return motion_project(p, c, b, lam);
+// Motions of kRows (even) vertically adjacent pixels of column x from row y0 on.
+template <int kRows>
+__device__ __forceinline__ void motion_column(const MotionParams &p, int x, int y0, float2 (&m)[kRows]) {
+    const MotionCol col = motion_col(p, x);
+    float2 b[kRows / 2], lam[kRows / 2];
+    bool ex[kRows], any = false;
+#pragma unroll
+    for (int r = 0; r < kRows; r += 2) {
+        b[r / 2] = motion_rows(p, y0 + r);
+        lam[r / 2] = motion_lambda(p, col, b[r / 2], &ex[r], &ex[r + 1]);
+        any = any || ex[r] || ex[r + 1];
+    }
+    if (any) {  // rare
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+            if (ex[r]) (r & 1 ? lam[r / 2].y : lam[r / 2].x) = entry_lambda_exact(p, x, y0 + r);
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; r += 2) {
+        const float4 q = motion_project(p, col, b[r / 2], lam[r / 2]);
+        m[r] = make_float2(q.x, q.y);
+        m[r + 1] = make_float2(q.z, q.w);
+    }
 }
 
+// Motions of kMotionRows vertically adjacent pixels of one column per thread:
+// the column terms are computed once and the rows' dependent chains (a
+// reciprocal square root and two reciprocals in series each) overlap; stores
+// stay coalesced along x.
+constexpr int kMotionRows = 4;
 __global__ void __launch_bounds__(256) motion_kernel(const __grid_constant__ MotionParams p,
                                                      float2 *__restrict__ motion) {
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
-    if (x >= p.width || y >= p.height) return;
-    motion[(size_t)y * p.width + x] = motion_at(p, x, y);
+    const int x = blockIdx.x * 32 + threadIdx.x;
+    const int y0 = (blockIdx.y * 8 + threadIdx.y) * kMotionRows;
+    if (x >= p.width || y0 >= p.height) return;
+    float2 m[kMotionRows];
+    motion_column<kMotionRows>(p, x, y0, m);
+#pragma unroll
+    for (int r = 0; r < kMotionRows; ++r)
+        if (y0 + r < p.height) motion[(size_t)(y0 + r) * p.width + x] = m[r];
 }
 
 __device__ __forceinline__ float4 load_hist(const float4 *h, size_t i) { return __ldg(h + i); }
@@ -193,59 +233,6 @@ __device__ __forceinline__ float4 blend4(float4 h, float4 c, float b) {
     const float2 xy = lerp2(make_float2(h.x, h.y), make_float2(c.x, c.y), b);
     const float2 zw = lerp2(make_float2(h.z, h.w), make_float2(c.z, c.w), b);
     return make_float4(xy.x, xy.y, zw.x, zw.y);
-}
-
-// TAA resolve (Sec. 3.2): reprojected, bilinearly filtered history clamped
-// to the current frame's 3x3 range, blended with the current frame.
-template <typename H>
-__global__ void __launch_bounds__(256) taa_kernel(const H *__restrict__ hist,
-                                                  const float4 *__restrict__ cur,
-                                                  const float2 *__restrict__ mot,
-                                                  H *__restrict__ out, int W, int Hh, float blend,
-                                                  unsigned *check) {
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
-    if (x >= W || y >= Hh) return;
-    const size_t i = (size_t)y * W + x;
-    const float4 c = __ldg(cur + i);
-    float4 res = c;
-    if (hist) {
-        const float2 m = __ldg(mot + i);
-        const float xc = (float)x + 0.5f, yc = (float)y + 0.5f;
-        // q = centre - m outside [0,W] x [0,H]: exact comparisons in FP32
-        const bool off = (m.x > xc) || (m.x < xc - (float)W) || (m.y > yc) || (m.y < yc - (float)Hh);
-        if (!off) {
-            // sample position (x - m.x, y - m.y) in texel-centre coordinates,
-            // split into integer and fraction without rounding
-            const float nx = -m.x, ny = -m.y;
-            const float flx = floorf(nx), fly = floorf(ny);
-            const float fx = nx - flx, fy = ny - fly;
-            const int ix = x + (int)flx, iy = y + (int)fly;
-            const int xa = min(max(ix, 0), W - 1), xb = min(max(ix + 1, 0), W - 1);
-            const int ya = min(max(iy, 0), Hh - 1), yb = min(max(iy + 1, 0), Hh - 1);
-            if (!in_range(check, xa >= 0 && xb < W && ya >= 0 && yb < Hh, kChkHistory)) return;
-            const float4 h00 = load_hist(hist, (size_t)ya * W + xa);
-            const float4 h01 = load_hist(hist, (size_t)ya * W + xb);
-            const float4 h10 = load_hist(hist, (size_t)yb * W + xa);
-            const float4 h11 = load_hist(hist, (size_t)yb * W + xb);
-            float4 h = bil4(fx, fy, h00, h01, h10, h11);
-            float4 mn = c, mx = c;
-#pragma unroll
-            for (int dy = -1; dy <= 1; ++dy) {
-                const int ny2 = min(max(y + dy, 0), Hh - 1);
-#pragma unroll
-                for (int dx = -1; dx <= 1; ++dx) {
-                    if (dx == 0 && dy == 0) continue;
-                    const int nx2 = min(max(x + dx, 0), W - 1);
-                    if (!in_range(check, nx2 >= 0 && nx2 < W && ny2 >= 0 && ny2 < Hh, kChkHistory)) continue;
-                    const float4 v = __ldg(cur + (size_t)ny2 * W + nx2);
-                    mn = fmin4(mn, v);
-                    mx = fmax4(mx, v);
-                }
-            }
-            res = blend4(fmin4(fmax4(h, mn), mx), c, blend);
-        }
-    }
-    store_hist(out, i, res);
 }
 
 // Reprojection and TAA resolve fused (Sec. 3.2): each pixel's motion is
@@ -311,15 +298,107 @@ __device__ __forceinline__ bool mbar_wait(const uint64_t *bar, unsigned parity, 
     return false;
 }
 
-// One 32x16-pixel tile (bx, by) of the fused resolve: the body of both the
-// single-view kernel and the multi-view kernel.  tile_map points to the
-// current frame's tensor map (kernel parameter or global memory), tile and bar
-// are the block's shared memory.
+// 16 bytes from global to shared memory, asynchronously (cp.async).
+__device__ __forceinline__ void copy_async16(void *smem, const void *global) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(smem)), "l"(global)
+                 : "memory");
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *p) {
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
+}
+
+// The history footprints of a thread's kPix vertically adjacent pixels, filtered
+// bilinearly: the off-screen test, then the texels around each sample position.
+template <typename H, int kPix>
+struct Footprints {
+    bool use[kPix];    // the pixel has history on screen
+    float4 hf[kPix];   // its filtered value
+
+    // mot(r, &m) gives the motion of pixel (x, y0 + r)
+    template <typename Motion>
+    __device__ __forceinline__ void gather(const H *__restrict__ hist, int x, int y0, int W, int Hh,
+                                           unsigned *check, const Motion &mot) {
+        float fxs[kPix], fys[kPix];
+        float4 h00[kPix], h01[kPix], h10[kPix], h11[kPix];
+#pragma unroll
+        for (int r = 0; r < kPix; ++r) {
+            use[r] = false;
+            const int y = y0 + r;
+            if (y >= Hh) continue;
+            const float2 m = mot(r);
+            const float xc = (float)x + 0.5f, yc = (float)y + 0.5f;
+            // q = centre - m outside [0,W] x [0,H]: exact comparisons in FP32
+            if ((m.x > xc) || (m.x < xc - (float)W) || (m.y > yc) || (m.y < yc - (float)Hh)) continue;
+            // sample position (x - m.x, y - m.y) in texel-centre coordinates,
+            // split into integer and fraction without rounding
+            const float nx = -m.x, ny = -m.y;
+            const float flx = floorf(nx), fly = floorf(ny);
+            fxs[r] = nx - flx;
+            fys[r] = ny - fly;
+            const int ix = x + (int)flx, iy = y + (int)fly;
+            const int xa = min(max(ix, 0), W - 1), xb = min(max(ix + 1, 0), W - 1);
+            const int ya = min(max(iy, 0), Hh - 1), yb = min(max(iy + 1, 0), Hh - 1);
+            if (!in_range(check, xa >= 0 && xb < W && ya >= 0 && yb < Hh, kChkHistory)) continue;
+            const H *ra = hist + (size_t)ya * W, *rb = hist + (size_t)yb * W;
+            h00[r] = load_hist(ra, xa);
+            h01[r] = load_hist(ra, xb);
+            h10[r] = load_hist(rb, xa);
+            h11[r] = load_hist(rb, xb);
+            use[r] = true;
+        }
+#pragma unroll
+        for (int r = 0; r < kPix; ++r)
+            if (use[r]) hf[r] = bil4(fxs[r], fys[r], h00[r], h01[r], h10[r], h11[r]);
+    }
+};
+
+template <int kPix>
+using ResolveTile = float4[8 * kPix + 2][kTW + 2];
+
+// The end of a resolved tile: 3x3 ranges from the kPix + 2 tile rows the
+// thread's windows cover (three-input min/max): each row's three texels reduced
+// once, each pixel combines three row results as soon as its last row is in;
+// clamp the filtered history, blend, store.
+template <typename H, int kPix>
+__device__ __forceinline__ void resolve_pixels(const ResolveTile<kPix> &tile, const Footprints<H, kPix> &f,
+                                               H *__restrict__ out, float blend, int x, int y0, int W,
+                                               int Hh, unsigned *check) {
+    constexpr int kTH = 8 * kPix;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    if (x >= W) return;
+    if (!in_range(check, tx + 2 < kTW + 2 && kPix * ty + kPix + 1 < kTH + 2, kChkTile)) return;
+    float4 rmn[kPix + 2], rmx[kPix + 2], cen[kPix + 2];
+#pragma unroll
+    for (int j = 0; j < kPix + 2; ++j) {
+        const float4 a = tile[kPix * ty + j][tx], b = tile[kPix * ty + j][tx + 1],
+                     d = tile[kPix * ty + j][tx + 2];
+        rmn[j] = min3_4(a, b, d);
+        rmx[j] = max3_4(a, b, d);
+        cen[j] = b;
+        if (j < 2) continue;
+        const int r = j - 2;  // the pixel whose window ends at row j
+        const int y = y0 + r;
+        if (y >= Hh) continue;
+        const float4 c = cen[r + 1];
+        float4 res = c;
+        if (f.use[r]) {
+            const float4 mn = min3_4(rmn[r], rmn[r + 1], rmn[r + 2]);
+            const float4 mx = max3_4(rmx[r], rmx[r + 1], rmx[r + 2]);
+            res = blend4(fmin4(fmax4(f.hf[r], mn), mx), c, blend);
+        }
+        if (in_range(check, y >= 0 && x >= 0, kChkPixel)) store_hist(out, (size_t)y * W + x, res);
+    }
+}
+
+// One tile (bx, by) of 32 x ResolvePix<H>::rows pixels of the fused resolve: the
+// body of both the single-view kernel and the multi-view kernel.  tile_map
+// points to the current frame's tensor map (kernel parameter or global memory),
+// tile and bar are the block's shared memory.
 template <typename H>
 __device__ __forceinline__ void resolve_tile(const CUtensorMap *tile_map, const MotionParams &mp,
                                              const H *__restrict__ hist, H *__restrict__ out,
-                                             float blend, int bx, int by,
-                                             float4 (&tile)[ResolvePix<H>::rows + 2][kTW + 2],
+                                             float blend, int bx, int by, ResolveTile<ResolvePix<H>::value> &tile,
                                              uint64_t &bar, int first_polls, unsigned int *status) {
     constexpr int kPix = ResolvePix<H>::value, kTH = ResolvePix<H>::rows;
     const int W = mp.width, Hh = mp.height;
@@ -335,6 +414,11 @@ __device__ __forceinline__ void resolve_tile(const CUtensorMap *tile_map, const 
     //    Thread 0 initialises the barrier and issues the copy; the other
     //    threads only touch the barrier after the __syncthreads below, so the
     //    motion arithmetic starts at once.
+    if (hist && x < W) {
+#pragma unroll
+        for (int r = 0; r < kPix; ++r)
+            if (y0 + kPix * ty + r < Hh) prefetch_l2(hist + (size_t)(y0 + kPix * ty + r) * W + x);
+    }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(&bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -350,51 +434,16 @@ __device__ __forceinline__ void resolve_tile(const CUtensorMap *tile_map, const 
     }
     // 2. motion (registers only) and the history footprint of the thread's
     //    pixels (rows kPix ty .. kPix ty + kPix - 1 of the tile): column terms
-    //    once, the pixels' arithmetic interleaved, the rare near-tie calls after
-    bool use[kPix];
-    float fxs[kPix], fys[kPix];
-    float4 h00[kPix], h01[kPix], h10[kPix], h11[kPix];
+    //    once, the pixels' arithmetic interleaved, the rare near-tie calls
+    //    after; filtered before the wait for the tile
+    Footprints<H, kPix> f;
 #pragma unroll
-    for (int r = 0; r < kPix; ++r) use[r] = false;
+    for (int r = 0; r < kPix; ++r) f.use[r] = false;
     if (hist && x < W) {
-        const MotionCol col = motion_col(mp, x);
-        float bs[kPix], lam[kPix];
-        bool ex[kPix];
-#pragma unroll
-        for (int r = 0; r < kPix; ++r) {
-            bs[r] = fmaf((float)(y0 + kPix * ty + r), mp.by, mp.b0);
-            lam[r] = motion_lambda(mp, col, bs[r], &ex[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < kPix; ++r)
-            if (ex[r]) lam[r] = entry_lambda_exact(mp, x, y0 + kPix * ty + r);
-#pragma unroll
-        for (int r = 0; r < kPix; ++r) {
-            const int y = y0 + kPix * ty + r;
-            if (y >= Hh) continue;
-            const float2 m = motion_project(mp, col, bs[r], lam[r]);
-            const float xc = (float)x + 0.5f, yc = (float)y + 0.5f;
-            if ((m.x > xc) || (m.x < xc - (float)W) || (m.y > yc) || (m.y < yc - (float)Hh)) continue;
-            const float nx = -m.x, ny = -m.y;
-            const float flx = floorf(nx), fly = floorf(ny);
-            fxs[r] = nx - flx;
-            fys[r] = ny - fly;
-            const int ix = x + (int)flx, iy = y + (int)fly;
-            const int xa = min(max(ix, 0), W - 1), xb = min(max(ix + 1, 0), W - 1);
-            const int ya = min(max(iy, 0), Hh - 1), yb = min(max(iy + 1, 0), Hh - 1);
-            if (!in_range(mp.check, xa >= 0 && xb < W && ya >= 0 && yb < Hh, kChkHistory)) continue;
-            const H *ra = hist + (size_t)ya * W, *rb = hist + (size_t)yb * W;
-            h00[r] = load_hist(ra, xa);
-            h01[r] = load_hist(ra, xb);
-            h10[r] = load_hist(rb, xa);
-            h11[r] = load_hist(rb, xb);
-            use[r] = true;
-        }
+        float2 m[kPix];
+        motion_column<kPix>(mp, x, y0 + kPix * ty, m);
+        f.gather(hist, x, y0 + kPix * ty, W, Hh, mp.check, [&](int r) { return m[r]; });
     }
-    float4 hf[kPix];  // filtered history, before the wait for the tile
-#pragma unroll
-    for (int r = 0; r < kPix; ++r)
-        if (use[r]) hf[r] = bil4(fxs[r], fys[r], h00[r], h01[r], h10[r], h11[r]);
     __syncthreads();  // the barrier's initialisation is visible to every thread
     const bool landed = mbar_wait(&bar, 0, first_polls);
     if (!__syncthreads_and(landed)) {
@@ -426,33 +475,65 @@ __device__ __forceinline__ void resolve_tile(const CUtensorMap *tile_map, const 
         }
         __syncthreads();
     }
-    if (x >= W) return;
-    if (!in_range(mp.check, tx + 2 < kTW + 2 && kPix * ty + kPix + 1 < kTH + 2, kChkTile)) return;
-    // 3. 3x3 ranges from the kPix + 2 tile rows the thread's windows cover
-    //    (three-input min/max): each row's three texels reduced once, each
-    //    pixel combines three row results as soon as its last row is in;
-    //    clamp the filtered history, blend
-    float4 rmn[kPix + 2], rmx[kPix + 2], cen[kPix + 2];
+    // 3. 3x3 ranges, clamp, blend
+    resolve_pixels<H, kPix>(tile, f, out, blend, x, y0 + kPix * ty, W, Hh, mp.check);
+}
+
+// TAA resolve (Sec. 3.2) with a given motion field: the pixel code of the fused
+// resolve; the current frame's tile, its halo clamped to the frame's edge, is
+// copied to shared memory asynchronously (cp.async) while the motion and then
+// the history footprints are read.  Bound by the latency of those two dependent
+// reads, so the motion is asked for first, the history's lines are prefetched
+// into the L2 without waiting for it (motion is a few pixels), and the smaller
+// tile of two pixels a thread lets four CTAs overlap: 1920x1080 FP32, motion
+// kernel included, 32.8 us against 40.6 us for one pixel a thread with its
+// neighbours read through L1.  Two pixels and 4 / 5 CTAs 34.7 / 34.6
+// us with the motion, four pixels and 3 CTAs 38.0, one pixel and 6 CTAs 38.1
+// (before the prefetch).
+constexpr int kTaaPix = 2, kTaaBlocks = 4;
+template <typename H>
+__global__ void __launch_bounds__(256, kTaaBlocks)
+    taa_kernel(const H *__restrict__ hist, const float4 *__restrict__ cur,
+               const float2 *__restrict__ mot, H *__restrict__ out, int W, int Hh, float blend,
+               unsigned *check) {
+    constexpr int kPix = kTaaPix, kTH = 8 * kPix;
+    __shared__ __align__(128) ResolveTile<kPix> tile;
+    const int x0 = blockIdx.x * kTW, y0 = blockIdx.y * kTH;
+    const int x = x0 + threadIdx.x, y = y0 + kPix * threadIdx.y;
+    float2 m[kPix];
+    if (hist) {
 #pragma unroll
-    for (int j = 0; j < kPix + 2; ++j) {
-        const float4 a = tile[kPix * ty + j][tx], b = tile[kPix * ty + j][tx + 1],
-                     d = tile[kPix * ty + j][tx + 2];
-        rmn[j] = min3_4(a, b, d);
-        rmx[j] = max3_4(a, b, d);
-        cen[j] = b;
-        if (j < 2) continue;
-        const int r = j - 2;  // the pixel whose window ends at row j
-        const int y = y0 + kPix * ty + r;
-        if (y >= Hh) continue;
-        const float4 c = cen[r + 1];
-        float4 res = c;
-        if (use[r]) {
-            const float4 mn = min3_4(rmn[r], rmn[r + 1], rmn[r + 2]);
-            const float4 mx = max3_4(rmx[r], rmx[r + 1], rmx[r + 2]);
-            res = blend4(fmin4(fmax4(hf[r], mn), mx), c, blend);
-        }
-        if (in_range(mp.check, y >= 0 && x >= 0, kChkPixel)) store_hist(out, (size_t)y * W + x, res);
+        for (int r = 0; r < kPix; ++r)
+            m[r] = x < W && y + r < Hh ? __ldg(mot + (size_t)(y + r) * W + x) : make_float2(0.0f, 0.0f);
     }
+    if (hist && x < W) {
+#pragma unroll
+        for (int r = 0; r < kPix; ++r)
+            if (y + r < Hh) prefetch_l2(hist + (size_t)(y + r) * W + x);
+    }
+    // row by row, a warp a row: texels -1 .. 30 of the row, then lanes 0 and 1
+    // the two to the right
+    const int xl = min(max(x - 1, 0), W - 1), xr = min(x + kTW - 1, W - 1);
+#pragma unroll
+    for (int k = 0; k <= kPix; ++k) {
+        const int r = threadIdx.y + 8 * k;
+        if (r >= kTH + 2) break;
+        const int yy = min(max(y0 + r - 1, 0), Hh - 1);
+        if (!in_range(check, xl < W && xr >= 0 && yy >= 0 && yy < Hh, kChkHistory)) continue;
+        const float4 *row = cur + (size_t)yy * W;
+        copy_async16(&tile[r][threadIdx.x], row + xl);
+        if (threadIdx.x < 2) copy_async16(&tile[r][threadIdx.x + kTW], row + xr);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    Footprints<H, kPix> f;
+#pragma unroll
+    for (int r = 0; r < kPix; ++r) f.use[r] = false;
+    if (hist && x < W) {
+        f.gather(hist, x, y, W, Hh, check, [&](int r) { return m[r]; });
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    resolve_pixels<H, kPix>(tile, f, out, blend, x, y, W, Hh, check);
 }
 
 template <typename H>
@@ -460,7 +541,7 @@ __global__ void __launch_bounds__(256, CLOUDVOL_TAA_MIN_BLOCKS)
     taa_reproject_kernel(const __grid_constant__ CUtensorMap tile_map,
                          const __grid_constant__ MotionParams mp, const H *__restrict__ hist,
                          H *__restrict__ out, float blend, int first_polls, unsigned int *status) {
-    __shared__ __align__(128) float4 tile[ResolvePix<H>::rows + 2][kTW + 2];
+    __shared__ __align__(128) ResolveTile<ResolvePix<H>::value> tile;
     __shared__ __align__(8) uint64_t bar;
     resolve_tile<H>(&tile_map, mp, hist, out, blend, blockIdx.x, blockIdx.y, tile, bar, first_polls,
                     status);
@@ -483,7 +564,7 @@ template <typename H>
 __global__ void __launch_bounds__(256, CLOUDVOL_TAA_MIN_BLOCKS)
     taa_reproject_batch_kernel(const ResolveView *__restrict__ views, int n_views, int first_polls,
                                unsigned int *status) {
-    __shared__ __align__(128) float4 tile[ResolvePix<H>::rows + 2][kTW + 2];
+    __shared__ __align__(128) ResolveTile<ResolvePix<H>::value> tile;
     __shared__ __align__(8) uint64_t bar;
     __shared__ MotionParams smp;
     __shared__ int s_view;
@@ -572,7 +653,7 @@ int launch_motion(const cloud_volume *vol, const cloud_params *prm, const cloud_
     if (!aligned(motion, 8)) return set_error(CLOUD_ERR_INVALID_ARG, "cloud_motion: motion not 8-byte aligned");
     MotionParams p;
     if (int rc = build_motion_params(vol, prm, prev, cur, width, height, &p)) return rc;
-    const dim3 grid((width + 31) / 32, (height + 7) / 8), block(32, 8);
+    const dim3 grid((width + 31) / 32, (height + 8 * kMotionRows - 1) / (8 * kMotionRows)), block(32, 8);
     motion_kernel<<<grid, block, 0, s>>>(p, (float2 *)motion);
     return check_launch("motion_kernel");
 }
@@ -596,7 +677,8 @@ int launch_taa(const void *history, const float *current, const float *motion, v
         if (a < b + px * eb && b < a + px * eb)
             return set_error(CLOUD_ERR_INVALID_ARG, "taa_resolve: history and history_out overlap");
     }
-    const dim3 grid((width + 31) / 32, (height + 7) / 8), block(32, 8);
+    const int rows = 8 * kTaaPix;
+    const dim3 grid((width + kTW - 1) / kTW, (height + rows - 1) / rows), block(32, 8);
     if (fmt == CLOUD_HISTORY_FP32)
         taa_kernel<float4><<<grid, block, 0, s>>>((const float4 *)history, (const float4 *)current,
                                                   (const float2 *)motion, (float4 *)history_out,

@@ -1,0 +1,50 @@
+"""GPU parity of the resolve kernels at the edges of their tiles: images one
+pixel short of, equal to and one past the tiles of 32x16 and 32x32 pixels, the
+separate motion and TAA passes against the FP64 oracle and the fused resolve
+bitwise against both, and the composite on both sides of its size rule.
+
+Tolerances: motion 1e-4 px, FP32 history 1e-6, FP16 history its storage rounding
+(2e-3 for values up to 2), composite 2e-6 (values up to 2)."""
+import numpy as np
+import pytest
+
+from paper_1609_05344_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1609_05344_gb300 import _native, api as A
+    _native.build()
+    return A
+
+
+def _t(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("w,h", [(31, 15), (32, 16), (33, 17), (32, 32), (65, 33), (2, 49), (97, 1)])
+@pytest.mark.parametrize("fmt", ["fp32", "fp16"])
+def test_tile_edges(api, oracle, w, h, fmt):
+    import torch
+    rng = np.random.default_rng(100 * w + h)
+    hist, cur = I.synthetic_frame(rng, h, w), I.synthetic_frame(rng, h, w)
+    hist = hist.astype(np.float16) if fmt == "fp16" else hist
+    mot = I.synthetic_motion(rng, h, w, offscreen_frac=0.1)
+    got = api.taa(_t(hist), _t(cur), _t(mot), history_fmt=fmt).cpu().numpy()
+    ref = oracle.taa(hist.astype(np.float64), cur, mot)
+    assert np.abs(got.astype(np.float64) - ref).max() <= (1e-6 if fmt == "fp32" else 2e-3)
+    # motion, and the fused resolve equal to motion followed by TAA
+    desc, prm = I.volume_desc("tiny", seed=1), I.params()
+    vol = api.Volume(desc)
+    prev, cam = I.orbit_camera(4, 3), I.orbit_camera(5, 3)
+    m = api.motion(vol, prm, prev, cam, w, h)
+    assert np.abs(m.cpu().numpy() - oracle.motion(desc, prm, prev, cam, w, h)).max() <= 1e-4
+    sep = api.taa(_t(hist), _t(cur), m, history_fmt=fmt)
+    fused = api.taa_reproject(vol, prm, prev, cam, _t(hist), _t(cur), history_fmt=fmt)
+    assert torch.equal(sep, fused)
