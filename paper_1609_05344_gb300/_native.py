@@ -8,6 +8,7 @@ from __future__ import annotations
 import concurrent.futures
 import ctypes
 import os
+import struct
 import subprocess
 import threading
 
@@ -205,6 +206,8 @@ _lib = None
 def lib():
     """The loaded library (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -244,12 +247,54 @@ def volume_desc(d: dict) -> VolumeDesc:
                       float(d.get("constant_density", 0.0)), PRECISION[d.get("precision", "fp32")])
 
 
+# One camera, parameter set and view as the C structures lay them out.  Filling
+# a structure from one packed buffer takes a third of the time of building it
+# field by field, which is most of a short call's host time; whatever does not
+# pack (a vector of another length, a number given as text) goes field by field.
+_CAMERA_PACK = struct.Struct("=13d")
+_PARAMS_PACK = struct.Struct("=14di4x")
+_VIEW_PACK = struct.Struct("=13d4iQ")
+assert _CAMERA_PACK.size == ctypes.sizeof(Camera) and _PARAMS_PACK.size == ctypes.sizeof(Params)
+assert _VIEW_PACK.size == ctypes.sizeof(View)
+_UNPACKABLE = (struct.error, TypeError, ValueError)
+
+
+def _camera_values(c: dict) -> tuple:
+    (px, py, pz), (fx, fy, fz) = c["pos"], c["forward"]
+    (rx, ry, rz), (ux, uy, uz) = c["right"], c["up"]
+    return px, py, pz, fx, fy, fz, rx, ry, rz, ux, uy, uz, c["tan_half_fovy"]
+
+
 def camera(c: dict) -> Camera:
-    return Camera(_D3(*c["pos"]), _D3(*c["forward"]), _D3(*c["right"]), _D3(*c["up"]),
-                  float(c["tan_half_fovy"]))
+    try:
+        return Camera.from_buffer_copy(_CAMERA_PACK.pack(*_camera_values(c)))
+    except _UNPACKABLE:
+        return Camera(_D3(*c["pos"]), _D3(*c["forward"]), _D3(*c["right"]), _D3(*c["up"]),
+                      float(c["tan_half_fovy"]))
 
 
 def params(p: dict) -> Params:
-    return Params(_D3(*p["sun_dir"]), _D3(*p["sun_radiance"]), _D3(*p["ambient"]), float(p["hg_g"]),
-                  float(p["absorption"]), float(p["light_step"]), float(p["tau_max"]),
-                  float(p["t_max"]), JITTER[p.get("jitter_mode", "pixel")])
+    try:
+        (sx, sy, sz), (er, eg, eb), (ar, ag, ab) = p["sun_dir"], p["sun_radiance"], p["ambient"]
+        return Params.from_buffer_copy(_PARAMS_PACK.pack(
+            sx, sy, sz, er, eg, eb, ar, ag, ab, p["hg_g"], p["absorption"], p["light_step"],
+            p["tau_max"], p["t_max"], JITTER[p.get("jitter_mode", "pixel")]))
+    except _UNPACKABLE:
+        return Params(_D3(*p["sun_dir"]), _D3(*p["sun_radiance"]), _D3(*p["ambient"]),
+                      float(p["hg_g"]), float(p["absorption"]), float(p["light_step"]),
+                      float(p["tau_max"]), float(p["t_max"]), JITTER[p.get("jitter_mode", "pixel")])
+
+
+def views(vs: list, outs: list):
+    """Array of View for view dictionaries and the device addresses of their outputs."""
+    try:
+        packed = b"".join([_VIEW_PACK.pack(*_camera_values(v["camera"]), v["width"], v["height"],
+                                           v["steps"], v.get("jitter_frame", -1), out)
+                           for v, out in zip(vs, outs)])
+        return (View * len(vs)).from_buffer_copy(packed)
+    except _UNPACKABLE:
+        arr = (View * len(vs))()
+        for i, v in enumerate(vs):
+            arr[i] = View(camera(v["camera"]), v["width"], v["height"], v["steps"],
+                          v.get("jitter_frame", -1), outs[i])
+        return arr

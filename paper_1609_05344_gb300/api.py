@@ -13,13 +13,16 @@ import torch
 from . import _native as N
 
 
-def _stream(stream=None) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream=None) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():  # the handle alone, without a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+def _ptr(t):
+    return None if t is None else t.data_ptr()
 
 
 def _require_cuda(t: torch.Tensor, name: str, dtype=None, shape=None):
@@ -27,7 +30,7 @@ def _require_cuda(t: torch.Tensor, name: str, dtype=None, shape=None):
     current device: anything else is refused here, before a launch."""
     if not isinstance(t, torch.Tensor) or not t.is_cuda or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous CUDA tensor")
-    if t.device.index != torch.cuda.current_device():
+    if t.get_device() != torch._C._cuda_getDevice():
         raise ValueError(f"{name} is on {t.device}, the current device is "
                          f"cuda:{torch.cuda.current_device()}")
     if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
@@ -398,11 +401,9 @@ class Batch:
                                            ctypes.byref(self._h)), "cloud_batch_create")
 
     def _array(self, views):
-        arr = (N.View * len(views))()
-        for i, v in enumerate(views):
-            arr[i] = N.View(N.camera(v["camera"]), v["width"], v["height"], v["steps"],
-                            v.get("jitter_frame", -1), self.outputs[i].data_ptr())
-        return arr
+        if len(views) > len(self.outputs):
+            raise IndexError("more views than the batch has outputs")
+        return N.views(views, [o.data_ptr() for o in self.outputs])
 
     def set_views(self, views: list, stream=None):
         arr = self._array(views)
