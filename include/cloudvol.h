@@ -310,7 +310,7 @@ int cloud_batch_autotune(cloud_batch *b, int repeats, float *times_ms, int *best
  * where cudaMalloc/cudaFree may block, synchronize the device or fail.
  * The caller still owns every view's out_rgba.  The scratch (work counter and
  * view table) is one library-wide static device array sized for
- * CLOUD_STATIC_MAX_VIEWS (256) views, 47360 bytes, which every GPU that loads
+ * CLOUD_STATIC_MAX_VIEWS (256) views, 57600 bytes, which every GPU that loads
  * the library holds until the process exits; n_views above 256 returns
  * CLOUD_ERR_INVALID_ARG.  The first call on a device looks up that array's
  * device address (a runtime query), so make it before any stream capture.

@@ -138,8 +138,11 @@ struct ViewParams {
     // Camera rays, unnormalised: v(x, y) = v00 + x vx + y vy, as double-float
     // pairs; vx/vy are split so that x * hi is exact (see split_df10).
     float v00h[3], v00l[3], vxh[3], vxl[3], vyh[3], vyl[3];
-    uint32_t org[kLatticeAxes];  // camera position in fixed-point lattice coordinates, half_unit taken off
-    uint32_t org_h;              // camera height above the layer bottom in 2^-16 m
+    // camera position in fixed-point lattice coordinates (half_unit taken off) and
+    // its height above the layer bottom in 2^-16 m, each as the nearest integer and
+    // the rest (in [-1/2, 1/2]): a sample's coordinate is rounded once, from the sum
+    uint32_t org[kLatticeAxes], org_h;
+    float org_rest[kLatticeAxes], org_h_rest;
     float zlo_h, zlo_l;    // slab_lo - o_z
     float zhi_h, zhi_l;    // slab_hi - o_z
     float tmax_h, tmax_l;  // far clip distance
@@ -185,6 +188,11 @@ constexpr int CHSizes[2] = {8, 16};
 constexpr int kConfigs = kShapes * 2;
 inline int config_shape(int config) { return config % kShapes; }
 inline int config_chunk(int config) { return CHSizes[(config / kShapes) & 1]; }
+// Step counts a march is compiled for: any, at most one chunk, more than one.
+// Single-view launches at the standard tile sizes know theirs (1920x1080 x 8
+// steps FP16 106.0 -> 103.4 us, 957x541 30.5 -> 30.1 us, four cameras' mean); the
+// views of a multi-view launch differ.
+enum StepRange { kAnySteps, kOneChunk, kManyChunks };
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
 // A ray's start coordinates and per-step increments as the warp stages them, in
@@ -415,7 +423,7 @@ __device__ __forceinline__ float step_depth(float absorption, float rho, float D
 // lookup is one whose density is exactly 0).  Returns the number of density
 // lookups this lane's ray performed in the method's sense (Sec. 1: one per
 // view step walked, plus the light steps of each step with density).
-template <typename T, int LS, int SHAPE, bool FX, int CH>
+template <typename T, int LS, int SHAPE, bool FX, int CH, int STEPS>
 __device__ __forceinline__ unsigned march_tile(
     const SceneParams &p, const ViewParams &v, int tile_x, int tile_y, WarpScratch<CH, FX> &ws,
     const T *__restrict__ base, const T *__restrict__ detail, const T *__restrict__ weather) {
@@ -511,13 +519,16 @@ __device__ __forceinline__ unsigned march_tile(
                     e[a] = e[a - kDX] * p.detail_mul;
                     continue;
                 }
-                const uint2 u = df2_to_u32(df2_mul_raw(pos[a < 6 ? a % 3 : a - 6], {p.kfix_h[a], p.kfix_l[a]}), wide);
+                df2 q = df2_mul_raw(pos[a < 6 ? a % 3 : a - 6], {p.kfix_h[a], p.kfix_l[a]});
+                q.lo.x += v.org_rest[a];
+                const uint2 u = df2_to_u32(q, wide);
                 c[a] = u.x + v.org[a];
                 e[a] = u.y;
             }
             // height above the layer bottom, in 2^-16 m
-            const uint2 uh = df2_to_u32({__fmul2_rn(pos[2].hi, both(65536.0f)),
-                                         __fmul2_rn(pos[2].lo, both(65536.0f))}, false);
+            df2 qh = {__fmul2_rn(pos[2].hi, both(65536.0f)), __fmul2_rn(pos[2].lo, both(65536.0f))};
+            qh.lo.x += v.org_h_rest;
+            const uint2 uh = df2_to_u32(qh, false);
             hq = (int32_t)(uh.x + v.org_h);
             eh = (int32_t)uh.y;
             const float vlen = n2f * rnf;
@@ -534,55 +545,91 @@ __device__ __forceinline__ unsigned march_tile(
     __syncwarp();
     const unsigned lt_mask = (1u << lane) - 1u;
     float tau = 0.0f, cr = 0.0f, cg = 0.0f, cb = 0.0f;
-    for (int i0 = 0; i0 < v.steps && __any_sync(kFull, alive); i0 += CH) {
+    constexpr int kScan = 16;  // steps per read of the grid in a march of many chunks
+    uint32_t occ_bits = 0;
+    int scanned = 0;
+    for (int i0 = 0; i0 < (STEPS == kOneChunk ? 1 : v.steps) && __any_sync(kFull, alive); i0 += CH) {
         const int nst = min(CH, v.steps - i0);
         // --- A1: which of this lane's CH steps need a density lookup: those in an
-        //     occupied macro-cell of the occupancy grid (the grid words of all CH
-        //     steps are loaded together, by every lane: the coordinates of a
-        //     finished ray and of steps past the last wrap into the grid too).  A
-        //     step outside the layer, possible only by rounding at the ends of the
-        //     clipped ray, is left to the lookup. -------------------------------
-        bool occ[CH];
-        if ((FX || !p.constant_mode) && p.occ) {
-            const uint4 s = ws.ray[lane][0], d = ws.ray[lane][1];
-            uint32_t bx = s.x + i0 * d.x, by = s.y + i0 * d.y, bz = s.z + i0 * d.z;
+        //     occupied macro-cell of the occupancy grid (the words of all steps are
+        //     loaded together, by every lane: the coordinates of a finished ray and
+        //     of steps past the last wrap into the grid too).  A step outside the
+        //     layer, possible only by rounding at the ends of the clipped ray, is
+        //     left to the lookup.
+        // --- A2: the warp's list of the (step, lane) lookups, to be shared out over
+        //     the lanes so that their loads overlap (a3) ---------------------------
+        const bool grid = (FX || !p.constant_mode) && p.occ;
+        uint32_t need = 0;
+        unsigned nq = 0;
+        const auto list = [&](int k, bool nd) {
+            const unsigned m = __ballot_sync(kFull, nd);
+            const unsigned slot = nq + __popc(m & lt_mask);
+            if (nd && in_range(p.check, slot < CH * 32u, kChkWork)) ws.pairs[slot] = (uint16_t)((k << 5) | lane);
+            nq += __popc(m);
+        };
+        if (STEPS == kManyChunks || (STEPS == kAnySteps && v.steps > CH)) {
+            // Long marches are mostly clear air, where the chain of grid reads is
+            // what takes time: two chunks' worth of steps per read, and one vote
+            // passes over them (or over one chunk) before any list is built.
+            // 1280x720 x 128 steps 494 -> 485 us, 64 views 10.25 -> 9.97 ms (kScan
+            // 32: 64 views 10.15 ms); the vote alone 378 -> 366 us, another view.
+            if (i0 >= scanned) {
+                scanned = i0 + kScan;
+                occ_bits = ~0u;
+                if (grid) {
+                    const uint4 s = ws.ray[lane][0], d = ws.ray[lane][1];
+                    uint32_t bx = s.x + i0 * d.x, by = s.y + i0 * d.y, bz = s.z + i0 * d.z;
+                    bool o[kScan];
 #pragma unroll
-            for (int k = 0; k < CH; ++k) {
-                occ[k] = occupied<FX>(p, bx, by, bz);
-                bx = mad32(d.x, p.one, bx);
-                by = mad32(d.y, p.one, by);
-                bz = mad32(d.z, p.one, bz);
+                    for (int k = 0; k < kScan; ++k) {
+                        o[k] = occupied<FX>(p, bx, by, bz);
+                        bx = mad32(d.x, p.one, bx);
+                        by = mad32(d.y, p.one, by);
+                        bz = mad32(d.z, p.one, bz);
+                    }
+                    occ_bits = 0;
+#pragma unroll
+                    for (int k = 0; k < kScan; ++k) occ_bits |= o[k] ? 1u << k : 0u;
+                }
+                const int left = v.steps - i0;
+                if (left < 32) occ_bits &= (1u << left) - 1u;
+                if (!__any_sync(kFull, alive && occ_bits)) {
+                    n_look += alive ? min(kScan, left) : 0;
+                    i0 += kScan - CH;
+                    continue;
+                }
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < CH; ++k) occ[k] = true;
-        }
-        // more than one chunk: most chunks of a long march are clear air warp-wide,
-        // which one vote settles before any list is built (1280x720 x 128 steps 378
-        // -> 366 us); a march of a single chunk almost never is (83.9 -> 84.4 us)
-        if (v.steps > CH) {
-            bool any = false;
-#pragma unroll
-            for (int k = 0; k < CH; ++k) any = any || (occ[k] && k < nst);
-            if (!__any_sync(kFull, any && alive)) {
+            need = alive ? occ_bits & ((1u << CH) - 1u) : 0u;
+            occ_bits >>= CH;
+            if (!__any_sync(kFull, need)) {
                 n_look += alive ? nst : 0;
                 continue;
             }
-        }
-        // --- A2: those (step, lane) lookups shared out over the warp, one or two
-        //     per lane at a time (ViewBatch) so that their loads overlap (a3) ---
-        uint32_t need = 0;
-        unsigned nq = 0;
 #pragma unroll
-        for (int k = 0; k < CH; ++k) {
-            const bool nd = occ[k] && alive && k < nst;
-            const unsigned m = __ballot_sync(kFull, nd);
-            const unsigned slot = nq + __popc(m & lt_mask);
-            if (nd) {
-                need |= 1u << k;
-                if (in_range(p.check, slot < CH * 32u, kChkWork)) ws.pairs[slot] = (uint16_t)((k << 5) | lane);
+            for (int k = 0; k < CH; ++k) list(k, (need >> k) & 1u);
+        } else {
+            // a march of one chunk: hardly ever clear, so straight to the list
+            bool o[CH];
+            if (grid) {
+                const uint4 s = ws.ray[lane][0], d = ws.ray[lane][1];
+                uint32_t bx = s.x + i0 * d.x, by = s.y + i0 * d.y, bz = s.z + i0 * d.z;
+#pragma unroll
+                for (int k = 0; k < CH; ++k) {
+                    o[k] = occupied<FX>(p, bx, by, bz);
+                    bx = mad32(d.x, p.one, bx);
+                    by = mad32(d.y, p.one, by);
+                    bz = mad32(d.z, p.one, bz);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < CH; ++k) o[k] = true;
             }
-            nq += __popc(m);
+#pragma unroll
+            for (int k = 0; k < CH; ++k) {
+                const bool nd = o[k] && alive && k < nst;
+                if (nd) need |= 1u << k;
+                list(k, nd);
+            }
         }
         if (nq == 0) {  // clear air, warp-wide: no optical depth, no early out
             n_look += alive ? nst : 0;

@@ -9,13 +9,13 @@
 
 namespace cloudvol {
 
-template <typename T, int LS, int SHAPE, bool FX, int CH>
+template <typename T, int LS, int SHAPE, bool FX, int CH, int STEPS>
 __global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
     march_kernel(const __grid_constant__ SceneParams p, const __grid_constant__ ViewParams v,
                  const T *__restrict__ base, const T *__restrict__ detail,
                  const T *__restrict__ weather, unsigned long long *__restrict__ counter) {
     __shared__ WarpScratch<CH, FX> scratch[4];
-    const unsigned n = march_tile<T, LS, SHAPE, FX, CH>(
+    const unsigned n = march_tile<T, LS, SHAPE, FX, CH, STEPS>(
         p, v, blockIdx.x, blockIdx.y, scratch[threadIdx.x >> 5], base, detail, weather);
     count_lookups(counter, n);
 }
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
         __syncthreads();
         const int local = t - sv.tile_begin;
         if (in_range(p.check, s_view >= 0 && s_view < n_views && local >= 0 && t < total_tiles, kChkView))
-            n_look += march_tile<T, LS, SHAPE, FX, CH>(p, sv, local % sv.tiles_x, local / sv.tiles_x,
+            n_look += march_tile<T, LS, SHAPE, FX, CH, kAnySteps>(p, sv, local % sv.tiles_x, local / sv.tiles_x,
                                                        scratch[threadIdx.x >> 5], base, detail, weather);
         __syncthreads();  // s_tile / sv are rewritten by the next iteration
     }
@@ -72,11 +72,12 @@ void launch_shape(const SceneParams &p, const ViewParams &v, const cloud_volume 
     const dim3 grid(v.tiles_x, (v.height + th - 1) / th);
     const T *b = (const T *)vol->base, *d = (const T *)vol->detail, *w = (const T *)vol->weather;
     if (fixed_sizes(p, vol))
-        march_kernel<T, 6, SHAPE, true, CH><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+        if (v.steps <= CH) march_kernel<T, 6, SHAPE, true, CH, kOneChunk><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+        else march_kernel<T, 6, SHAPE, true, CH, kManyChunks><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
     else if (p.light_steps == 6)
-        march_kernel<T, 6, SHAPE, false, CH><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+        march_kernel<T, 6, SHAPE, false, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
     else
-        march_kernel<T, -1, SHAPE, false, CH><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+        march_kernel<T, -1, SHAPE, false, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
 }
 
 template <typename T, int CH>

@@ -148,11 +148,14 @@ int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_cam
         for (int a = 0; a < kLatticeAxes; ++a) {
             if (L[a] == 0) continue;  // absent tile: axis unused
             const double t = cam->pos[a < 6 ? a % 3 : a - 6] / P[a];
-            v->org[a] = (uint32_t)(unsigned long long)std::llrint((t - std::floor(t)) * 4294967296.0) -
-                        (1u << (31 - L[a]));
+            const double units = (t - std::floor(t)) * 4294967296.0, whole = std::nearbyint(units);
+            v->org[a] = (uint32_t)(unsigned long long)whole - (1u << (31 - L[a]));
+            v->org_rest[a] = (float)(units - whole);
         }
     }
-    v->org_h = (uint32_t)(unsigned long long)std::llrint((cam->pos[2] - d.slab_lo_m) * 65536.0);
+    const double above = (cam->pos[2] - d.slab_lo_m) * 65536.0;
+    v->org_h = (uint32_t)(unsigned long long)std::llrint(above);
+    v->org_h_rest = (float)(above - std::nearbyint(above));
     split_df(d.slab_lo_m - cam->pos[2], &v->zlo_h, &v->zlo_l);
     split_df(d.slab_hi_m - cam->pos[2], &v->zhi_h, &v->zhi_l);
     split_df(prm->t_max_m, &v->tmax_h, &v->tmax_l);
