@@ -23,7 +23,7 @@ CHECKED_BUILD_DIR = os.path.join(_HERE, "_build_checked")
 CHECKED_LIB_PATH = os.path.join(_HERE, "libcloudvol_checked.so")
 HEADER = os.path.join(_ROOT, "include", "cloudvol.h")
 SOURCES = ["volume.cu", "render.cu", "batch.cu", "march8_view.cu", "march16_view.cu",
-           "march8_batch.cu", "march16_batch.cu", "taa.cu", "session.cu", "server.cu"]
+           "march8_batch.cu", "march16_batch.cu", "march_small.cu", "taa.cu", "session.cu", "server.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", ARCH, "-Xcompiler", "-fPIC", "-Xptxas", "-v",
               "--expt-relaxed-constexpr"]

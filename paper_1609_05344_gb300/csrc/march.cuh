@@ -163,7 +163,13 @@ struct ViewParams {
 //   shape 1: warp 8x4,  CTA 4x1 warps -> 32x4 pixels
 //   shape 2: warp 16x2, CTA 2x2 warps -> 32x4 pixels
 //   shape 3: warp 4x8,  CTA 2x2 warps -> 8x16 pixels
-constexpr int kShapes = 4;
+// and three with fewer rays than lanes, for images that would not fill the GPU
+// (small_shape in render.cu): the shared-out phases still use every lane
+//   shape 4: warp 4x4,  CTA 2x2 warps -> 8x8 pixels
+//   shape 5: warp 4x2,  CTA 2x2 warps -> 8x4 pixels
+//   shape 6: warp 2x2,  CTA 2x2 warps -> 4x4 pixels
+constexpr int kShapes = 4;  // those the autotuner chooses from
+constexpr int kAllShapes = 7;
 template <int S>
 struct TileShape;
 template <>
@@ -174,8 +180,14 @@ template <>
 struct TileShape<2> { static constexpr int WX = 16, WY = 2, CX = 2, CY = 2; };
 template <>
 struct TileShape<3> { static constexpr int WX = 4, WY = 8, CX = 2, CY = 2; };
+template <>
+struct TileShape<4> { static constexpr int WX = 4, WY = 4, CX = 2, CY = 2; };
+template <>
+struct TileShape<5> { static constexpr int WX = 4, WY = 2, CX = 2, CY = 2; };
+template <>
+struct TileShape<6> { static constexpr int WX = 2, WY = 2, CX = 2, CY = 2; };
 inline void tile_dims(int shape, int *tw, int *th) {
-    static const int w[kShapes] = {16, 32, 32, 8}, h[kShapes] = {8, 4, 4, 16};
+    static const int w[kAllShapes] = {16, 32, 32, 8, 8, 8, 4}, h[kAllShapes] = {8, 4, 4, 16, 8, 4, 4};
     *tw = w[shape];
     *th = h[shape];
 }
@@ -431,7 +443,7 @@ __device__ __forceinline__ unsigned march_tile(
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int x = tile_x * (S::WX * S::CX) + (warp % S::CX) * S::WX + (lane % S::WX);
     const int y = tile_y * (S::WY * S::CY) + (warp / S::CX) * S::WY + (lane / S::WX);
-    const bool in_image = x < v.width && y < v.height;
+    const bool in_image = lane < S::WX * S::WY && x < v.width && y < v.height;
     bool inside = in_image;
     const int nlight = LS >= 0 ? LS : p.light_steps;
     unsigned n_look = 0;
@@ -775,6 +787,9 @@ int launch_march(const SceneParams &p, const ViewParams &v, const cloud_volume *
 template <int CH>
 void launch_march_ch(const SceneParams &p, const ViewParams &v, const cloud_volume *vol,
                      unsigned long long *counter, int shape, cudaStream_t s);
+// The same with the small shapes (4, 5, 6) and 8 view steps a chunk (march_small.cu).
+void launch_march_small(const SceneParams &p, const ViewParams &v, const cloud_volume *vol,
+                        unsigned long long *counter, int shape, cudaStream_t s);
 template <int CH>
 const void *batch_kernel_ch(int precision, int light_steps, bool fx, int shape);
 // True when a launch can use the FX march: the standard tile sizes, all three

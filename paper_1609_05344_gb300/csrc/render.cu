@@ -209,6 +209,20 @@ void set_tuned_config(int precision, int light_steps, int config) {
     g_best_config[precision & 3][light_steps == 6 ? 1 : 0] = config;
 }
 
+// Tile shape of a single view too small to fill the GPU, or -1.  Below one wave
+// of warps (32 on each of the 152 SMs) a launch is a chain of latencies, shorter
+// the fewer rays share a warp's lookups: 8 or 16 rays a warp while that still
+// fits one wave, 4 up to half a wave (their setup wastes more lanes than it
+// gains beyond).  GPU time, 32 / 16 / 8 / 4 rays a warp, 64 steps, FP32, full
+// tiles: 64x64 62.0 / 44.7 / 32.4 / 28.9 us, 128x128 69.5 / 46.3 / 35.0 / 35.6,
+// 200x160 71.2 / 50.3 / 41.0 / 53.2, 320x240 78.4 / 60.3 / 69.6 / 92.3; 8 steps:
+// 9.9 / 7.9 / 5.9 / 5.9, 11.3 / 8.2 / 6.8 / 8.5, 11.7 / 9.1 / 8.9 / 13.0, 13.2 /
+// 11.9 / 15.6 / 23.7; 640x360 x 8 steps 23.1 / 24.9 / 35.8.
+static int small_shape(int width, int height) {
+    const int64_t wave = 152 * 32, pixels = (int64_t)width * height;
+    return pixels <= 2 * wave ? 6 : pixels <= 8 * wave ? 5 : pixels <= 16 * wave ? 4 : -1;
+}
+
 bool fixed_sizes(const SceneParams &p, const cloud_volume *vol) {
     return p.light_steps == 6 && !p.constant_mode && vol->detail && vol->weather &&
            p.log2_base == kStdLog2Base && p.log2_detail == kStdLog2Detail &&
@@ -233,12 +247,14 @@ int launch_render(const cloud_volume *vol, const cloud_camera *cam, const cloud_
         return set_error(CLOUD_ERR_INVALID_ARG, "cloud_render: counter not 8-byte aligned");
     SceneParams p;
     ViewParams v;
-    const int config = tuned_config(vol->desc.precision, light_steps);
+    const int config = tuned_config(vol->desc.precision, light_steps), small = small_shape(width, height);
     if (int rc = build_scene(vol, prm, light_steps, integration, &p)) return rc;
     if (int rc = build_view(vol, prm, cam, width, height, steps, jitter_frame, out,
-                            config_shape(config), &v))
+                            small >= 0 ? small : config_shape(config), &v))
         return rc;
-    return launch_march(p, v, vol, counter, config, s);
+    if (small < 0) return launch_march(p, v, vol, counter, config, s);
+    launch_march_small(p, v, vol, counter, small, s);
+    return check_launch("march_kernel");
 }
 
 }  // namespace cloudvol

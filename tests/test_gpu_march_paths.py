@@ -66,9 +66,28 @@ def test_partial_and_clear_chunks(api, oracle, steps, config):
     api.set_launch_config("fp32", 6, config)
     try:
         cam = I.camera((0.0, 0.0, 500.0), 70.0, 36.0, 60.0)
-        ref, count, n = _check(api, oracle, desc, I.params(), cam, 33, 18, steps, 6)
+        ref, count, n = _check(api, oracle, desc, I.params(), cam, 330, 240, steps, 6)
     finally:
         api.set_launch_config("fp32", 6, 3)
     # lookups in the method's sense: a density within rounding of 0, or an optical depth
     # within rounding of the early out, may move single steps of single rays
     assert abs(count - n) <= 1e-3 * n + 6
+
+
+# the edges of the rule that spreads small images over more warps (4, 8, 16 and 32 rays each):
+# 9728, 38912 and 77824 pixels, ragged against every tile; the multi-view launch always has 32
+@pytest.mark.parametrize("w,h", [(1, 1), (5, 3), (64, 152), (97, 101), (256, 152), (261, 151), (304, 256),
+                                 (307, 257)])
+@pytest.mark.parametrize("kind,precision", [("full", "fp32"), ("full", "bf16"), ("tiny", "fp32"),
+                                            ("tiny", "unorm16")])
+@pytest.mark.parametrize("steps", [8, 21])
+def test_small_images_equal_batched_views(api, w, h, kind, precision, steps):
+    import torch
+    vol = api.Volume(I.volume_desc(kind, seed=8, precision=precision))
+    cam = I.camera((100.0, -700.0, 500.0), 210.0, 36.0, 60.0)
+    view = dict(camera=cam, width=w, height=h, steps=steps, jitter_frame=5)
+    for light_steps in (6, 3):
+        one, count = api.render(vol, cam, I.params(), w, h, steps, light_steps, jitter_frame=5, count=True)
+        batch = api.Batch(vol, I.params(), [view], light_steps)
+        assert torch.equal(one, batch.render()[0])
+        assert int(count.item()) >= int((one[..., 3] > 0).sum().item())
