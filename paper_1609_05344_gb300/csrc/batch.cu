@@ -20,10 +20,9 @@
 
 namespace cloudvol {
 
-static const void *batch_kernel(int precision, int light_steps, bool fx, int config) {
-    return config_chunk(config) == 16
-               ? batch_kernel_ch<16>(precision, light_steps, fx, config_shape(config))
-               : batch_kernel_ch<8>(precision, light_steps, fx, config_shape(config));
+static const void *batch_kernel(int precision, int kind, int config) {
+    return config_chunk(config) == 16 ? batch_kernel_ch<16>(precision, kind, config_shape(config))
+                                      : batch_kernel_ch<8>(precision, kind, config_shape(config));
 }
 
 // Enqueue counter reset + persistent kernel for the given table on stream s.
@@ -31,7 +30,7 @@ int launch_batch(const cloud_volume *vol, const SceneParams &scene, const ViewPa
                  int n_views, int total_tiles, int config, unsigned int *d_work,
                  unsigned long long *counter, cudaStream_t s) {
     if (total_tiles == 0) return CLOUD_OK;
-    const void *fn = batch_kernel(vol->desc.precision, scene.light_steps, fixed_sizes(scene, vol), config);
+    const void *fn = batch_kernel(vol->desc.precision, volume_kind(scene, vol), config);
     int dev = 0, sms = 0, per_sm = 0;
     if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
     if (int rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev),

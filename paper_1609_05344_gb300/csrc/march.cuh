@@ -19,12 +19,14 @@
 #include "common.cuh"
 
 // CTAs per SM the march is compiled for (register budget 65536 / (128 x this)),
-// for FP32 records and for 16-bit records (which need fewer registers).
+// for FP32 records and for 16-bit records (which need fewer registers): volumes of
+// any tile sizes (64^3 base, 1280x720 x 64 steps: 234.4 us against 242.6 with 5;
+// FP16 236.7 against 243.7 with 6).
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_F32
-#define CLOUDVOL_MARCH_MIN_BLOCKS_F32 5
+#define CLOUDVOL_MARCH_MIN_BLOCKS_F32 6
 #endif
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_16
-#define CLOUDVOL_MARCH_MIN_BLOCKS_16 6
+#define CLOUDVOL_MARCH_MIN_BLOCKS_16 7
 #endif
 
 namespace cloudvol {
@@ -47,17 +49,24 @@ namespace cloudvol {
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16
 #define CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16 6
 #endif
-template <typename T, bool FX, int CH>
+// What a march is compiled for: any volume; the standard tile sizes (below); a
+// base tile of any size alone, with neither detail nor weather, which needs a
+// third of the records and registers for 8 CTAs (64^3 base, 1280x720 x 64 steps
+// 520.7 us as any volume, 307.5 as this).  The number of light steps is a launch
+// value: compiled in, it gained nothing, and kept standard volumes with other
+// than six light steps (nine: 480 -> 431 us) from their own kernel.
+enum VolumeKind { kAnyVolume, kStandardVolume, kBaseVolume };
+template <typename T, int VOL, int CH>
 struct MarchBlocks {
     static constexpr bool f32 = sizeof(T) == 4;
     static constexpr int value =
-        !FX ? (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32 : CLOUDVOL_MARCH_MIN_BLOCKS_16)
+        VOL == kAnyVolume ? (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32 : CLOUDVOL_MARCH_MIN_BLOCKS_16)
         : CH <= 8 ? (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX : CLOUDVOL_MARCH_MIN_BLOCKS_16_FX)
                   : (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX16 : CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16);
 };
 
 // The standard tile sizes (128^3 base, 32^3 detail, 512^2 weather records) as
-// compile-time constants: with FX the record-index and weight shifts of every
+// compile-time constants: the record-index and weight shifts of every
 // lookup are immediates instead of per-launch values.
 constexpr int kStdLog2Base = 7, kStdLog2Detail = 5, kStdLog2Weather = 9;
 
@@ -65,16 +74,22 @@ constexpr int kStdLog2Base = 7, kStdLog2Detail = 5, kStdLog2Weather = 9;
 // density code is inlined that many times): one for FP32 records, whose three
 // wide loads per sample keep the memory busy (1920x1080 x 8 steps 86.1 us, two
 // 86.8, three 96.9); two for 16-bit ones (64 views 10.86 ms, one 11.38, three
-// 11.11) and where the tile sizes are not constants.
+// 11.11) and where the tile sizes are not constants; three for a base tile alone,
+// one record a sample (1280x720 x 64 steps 307.5 us, one 339.6, two 313.7, six
+// 305.6; 128x128 32.3, 39.2, 33.3, 33.1).
 #ifndef CLOUDVOL_LIGHT_UNROLL_F32
 #define CLOUDVOL_LIGHT_UNROLL_F32 1
+#endif
+#ifndef CLOUDVOL_LIGHT_UNROLL_BASE
+#define CLOUDVOL_LIGHT_UNROLL_BASE 3
 #endif
 #ifndef CLOUDVOL_LIGHT_UNROLL_16
 #define CLOUDVOL_LIGHT_UNROLL_16 2
 #endif
-template <typename T, bool FX>
+template <typename T, int VOL>
 struct LightUnroll {
-    static constexpr int value = FX && sizeof(T) == 4 ? CLOUDVOL_LIGHT_UNROLL_F32 : CLOUDVOL_LIGHT_UNROLL_16;
+    static constexpr int value = VOL == kBaseVolume                             ? CLOUDVOL_LIGHT_UNROLL_BASE
+                                 : VOL == kStandardVolume && sizeof(T) == 4 ? CLOUDVOL_LIGHT_UNROLL_F32 : CLOUDVOL_LIGHT_UNROLL_16;
 };
 // View lookups a lane evaluates per round of the shared-out view phase (their
 // record loads can overlap; more of them cost registers): one for FP32
@@ -208,27 +223,28 @@ enum StepRange { kAnySteps, kOneChunk, kManyChunks };
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
 // A ray's start coordinates and per-step increments as the warp stages them, in
-// 16-byte groups so that a lane fetches another lane's ray with three (FX) or
+// 16-byte groups so that a lane fetches another lane's ray with two, three or
 // five wide shared loads instead of one load per axis:
 //   group 0  start of base x, y, z and of the height
 //   group 1  their increments
 //   group 2  start of weather x, y, then their increments
 //   group 3  start of detail x, y, z, then the increment of detail x
 //   group 4  increments of detail y, z
-// FX (the base tile period is 2^detail_shift detail periods) has no groups 3
-// and 4: the detail coordinates follow from the base ones by an exact shift.
+// Standard volumes (the base tile period is 2^detail_shift detail periods) have no
+// groups 3 and 4: the detail coordinates follow from the base ones by an exact
+// shift; a base tile alone uses groups 0 and 1.
 // Three and five groups a lane are odd strides: lanes that fetch neighbouring
 // rays meet no bank conflict.
-template <bool FX>
-struct RayGroups { static constexpr int value = FX ? 3 : 5; };
+template <int VOL>
+struct RayGroups { static constexpr int value = VOL == kAnyVolume ? 5 : 3; };
 
 // Per-warp shared scratch of the march: each lane's staged ray and step length,
 // the list of (step, lane) pairs to evaluate, and two values per (step, lane)
 // of a chunk of CH view steps: the view density, then the integration weight;
 // the optical depth before the step, then the sun's share of the light.
-template <int CH, bool FX>
+template <int CH, int VOL>
 struct WarpScratch {
-    uint4 ray[32][RayGroups<FX>::value];
+    uint4 ray[32][RayGroups<VOL>::value];
     float length[32];
     float rho[CH][32];
     float aux[CH][32];
@@ -293,10 +309,10 @@ __device__ __forceinline__ float height_profile(const SceneParams &p, int32_t hq
 // standard sizes a cell coordinate is the top byte of the base coordinate, so
 // two byte permutations gather the cell index and its low bits select the bit
 // (the funnel shift takes its count modulo 32).
-template <bool FX>
+template <int VOL>
 __device__ __forceinline__ bool occupied(const SceneParams &p, uint32_t bx, uint32_t by, uint32_t bz) {
     // macro-cell = record index >> kOccShift on each axis; bits x fastest
-    constexpr bool kBytes = FX && kStdLog2Base - kOccShift == 8;
+    constexpr bool FX = VOL == kStandardVolume, kBytes = FX && kStdLog2Base - kOccShift == 8;
     const int lo = FX ? kStdLog2Base - kOccShift : p.log2_occ, sh = 32 - lo;
     const uint32_t cell = kBytes ? __byte_perm(__byte_perm(bx, by, 0x7373), bz >> 24, 0x5410)
                                  : ((bz >> sh) << (2 * lo)) | ((by >> sh) << lo) | (bx >> sh);
@@ -319,86 +335,94 @@ struct Density {
     float gw, r;
     __device__ __forceinline__ float value() const { return __fmul_rn(gw, r); }
 };
-template <bool FX, typename T>
+template <int VOL, typename T>
 __device__ __forceinline__ Density density(const SceneParams &p, const T *__restrict__ base,
                                            const T *__restrict__ detail,
                                            const T *__restrict__ weather, const uint32_t c[8],
                                            int32_t hq) {
+    constexpr bool FX = VOL == kStandardVolume;
+    const bool has_detail = FX || (VOL == kAnyVolume && detail), has_weather = FX || (VOL == kAnyVolume && weather);
     const int lb = FX ? kStdLog2Base : p.log2_base, ld = FX ? kStdLog2Detail : p.log2_detail,
               lw = FX ? kStdLog2Weather : p.log2_weather;
-    if (!FX && p.constant_mode) return {p.rho0, 1.0f};
+    if (VOL == kAnyVolume && p.constant_mode) return {p.rho0, 1.0f};
     const float g = height_profile(p, hq);
     float cb[8], cd[8], cw[4];
     const uint32_t rb = rec3(p.base_mul, lb, c[kBX], c[kBY], c[kBZ]),
                    rd = rec3(p.detail_rec_mul, ld, c[kDX], c[kDY], c[kDZ]),
                    rw = rec2(p.weather_mul, lw, c[kWX], c[kWY]);
     if (!in_range(p.check,
-                  rb < (1u << (3 * lb)) && (!(FX || detail) || rd < (1u << (3 * ld))) &&
-                      (!(FX || weather) || rw < (1u << (2 * lw))),
+                  rb < (1u << (3 * lb)) && (!has_detail || rd < (1u << (3 * ld))) &&
+                      (!has_weather || rw < (1u << (2 * lw))),
                   kChkRecord))
         return {0.0f, 0.0f};
     const float ob = load_rec8(base, rb, cb);
     float od = 0.0f, ow = 0.0f;
-    if (FX || detail) od = load_rec8(detail, rd, cd);
-    if (FX || weather) ow = load_rec4(weather, rw, cw);
+    if (has_detail) od = load_rec8(detail, rd, cd);
+    if (has_weather) ow = load_rec4(weather, rw, cw);
     const float2 fb = frac23(c[kBX] << lb, c[kBY] << lb), fd = frac23(c[kDX] << ld, c[kDY] << ld),
                  fz = frac23(c[kBZ] << lb, c[kDZ] << ld), fw = frac23(c[kWX] << lw, c[kWY] << lw);
     const float b = trilerp(cb, fb.x, fb.y, fz.x) + ob;
     float r = b + p.k0;
-    if (FX || detail) {
+    if (has_detail) {
         const float dt = trilerp(cd, fd.x, fd.y, fz.y) + od;
         r = fmaf(-p.detail_w, dt, r);
     }
     r = fmaxf(r * p.inv_1mc, 0.0f);
-    const float w = (FX || weather) ? bilerp(cw, fw.x, fw.y) + ow + p.w_off : 1.0f;
+    const float w = has_weather ? bilerp(cw, fw.x, fw.y) + ow + p.w_off : 1.0f;
     return {__fmul_rn(g, w), r};
 }
 
-// Coordinates of light sample j of a point (FX: the detail coordinates follow
-// from the base ones).
-template <bool FX>
+// Coordinates of light sample j of a point (standard volumes: the detail
+// coordinates follow from the base ones).
+template <int VOL>
 __device__ __forceinline__ void light_coords(const SceneParams &p, const uint32_t cs[kLatticeAxes], int j,
                                              uint32_t cj[kLatticeAxes]) {
 #pragma unroll
     for (int a = 0; a < kLatticeAxes; ++a)
-        cj[a] = FX && a >= kDX && a <= kDZ ? mad32(cj[a - kDX], p.detail_mul, p.detail_add)
+        cj[a] = VOL == kStandardVolume && a >= kDX && a <= kDZ ? mad32(cj[a - kDX], p.detail_mul, p.detail_add)
                                            : mad32(cs[a], p.one, p.loff[j][a]);
 }
 
 // Staging of one lane's start coordinates and increments (lattice axes, then
 // the height) into the warp's scratch.
-template <int CH, bool FX>
-__device__ __forceinline__ void stage_ray(WarpScratch<CH, FX> &ws, unsigned lane,
+template <int CH, int VOL>
+__device__ __forceinline__ void stage_ray(WarpScratch<CH, VOL> &ws, unsigned lane,
                                           const uint32_t c[kLatticeAxes],
                                           const uint32_t e[kLatticeAxes], int32_t hq, int32_t eh) {
     ws.ray[lane][0] = make_uint4(c[kBX], c[kBY], c[kBZ], (uint32_t)hq);
     ws.ray[lane][1] = make_uint4(e[kBX], e[kBY], e[kBZ], (uint32_t)eh);
-    ws.ray[lane][2] = make_uint4(c[kWX], c[kWY], e[kWX], e[kWY]);
-    if (!FX) {
-        ws.ray[lane][RayGroups<FX>::value - 2] = make_uint4(c[kDX], c[kDY], c[kDZ], e[kDX]);
-        ws.ray[lane][RayGroups<FX>::value - 1] = make_uint4(e[kDY], e[kDZ], 0u, 0u);
+    if (VOL != kBaseVolume) ws.ray[lane][2] = make_uint4(c[kWX], c[kWY], e[kWX], e[kWY]);
+    if (VOL == kAnyVolume) {
+        ws.ray[lane][RayGroups<VOL>::value - 2] = make_uint4(c[kDX], c[kDY], c[kDZ], e[kDX]);
+        ws.ray[lane][RayGroups<VOL>::value - 1] = make_uint4(e[kDY], e[kDZ], 0u, 0u);
     }
 }
 
 // Coordinates of view step i of ray `ow` of the warp from its staged start and
 // increment (integer arithmetic: the same values as adding the increment step
-// by step; for FX the detail coordinates are the base ones shifted exactly,
+// by step; in standard volumes the detail coordinates are the base ones shifted,
 // as the ray setup derives them).  Returns the height.
-template <int CH, bool FX>
-__device__ __forceinline__ int32_t step_coords(const SceneParams &p, const WarpScratch<CH, FX> &ws,
+template <int CH, int VOL>
+__device__ __forceinline__ int32_t step_coords(const SceneParams &p, const WarpScratch<CH, VOL> &ws,
                                                unsigned ow, uint32_t i, uint32_t cs[kLatticeAxes]) {
-    const uint4 s = ws.ray[ow][0], e = ws.ray[ow][1], w = ws.ray[ow][2];
+    const uint4 s = ws.ray[ow][0], e = ws.ray[ow][1];
     cs[kBX] = s.x + i * e.x;
     cs[kBY] = s.y + i * e.y;
     cs[kBZ] = s.z + i * e.z;
+    if (VOL == kBaseVolume) {
+#pragma unroll
+        for (int a = kDX; a < kLatticeAxes; ++a) cs[a] = 0u;  // no such tile
+        return (int32_t)(s.w + i * e.w);
+    }
+    const uint4 w = ws.ray[ow][2];
     cs[kWX] = w.x + i * w.z;
     cs[kWY] = w.y + i * w.w;
-    if (FX) {
+    if (VOL == kStandardVolume) {
 #pragma unroll
         for (int b = 0; b < 3; ++b)
             cs[kDX + b] = mad32(cs[b], p.detail_mul, p.detail_add);
     } else {
-        const uint4 d = ws.ray[ow][RayGroups<FX>::value - 2], f = ws.ray[ow][RayGroups<FX>::value - 1];
+        const uint4 d = ws.ray[ow][RayGroups<VOL>::value - 2], f = ws.ray[ow][RayGroups<VOL>::value - 1];
         cs[kDX] = d.x + i * d.w;
         cs[kDY] = d.y + i * f.x;
         cs[kDZ] = d.z + i * f.y;
@@ -435,9 +459,9 @@ __device__ __forceinline__ float step_depth(float absorption, float rho, float D
 // lookup is one whose density is exactly 0).  Returns the number of density
 // lookups this lane's ray performed in the method's sense (Sec. 1: one per
 // view step walked, plus the light steps of each step with density).
-template <typename T, int LS, int SHAPE, bool FX, int CH, int STEPS>
+template <typename T, int SHAPE, int VOL, int CH, int STEPS>
 __device__ __forceinline__ unsigned march_tile(
-    const SceneParams &p, const ViewParams &v, int tile_x, int tile_y, WarpScratch<CH, FX> &ws,
+    const SceneParams &p, const ViewParams &v, int tile_x, int tile_y, WarpScratch<CH, VOL> &ws,
     const T *__restrict__ base, const T *__restrict__ detail, const T *__restrict__ weather) {
     using S = TileShape<SHAPE>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -445,7 +469,7 @@ __device__ __forceinline__ unsigned march_tile(
     const int y = tile_y * (S::WY * S::CY) + (warp / S::CX) * S::WY + (lane / S::WX);
     const bool in_image = lane < S::WX * S::WY && x < v.width && y < v.height;
     bool inside = in_image;
-    const int nlight = LS >= 0 ? LS : p.light_steps;
+    const int nlight = p.light_steps;
     unsigned n_look = 0;
     uint32_t c[kLatticeAxes] = {}, e[kLatticeAxes] = {};
     int32_t hq = 0, eh = 0;
@@ -570,7 +594,7 @@ __device__ __forceinline__ unsigned march_tile(
         //     left to the lookup.
         // --- A2: the warp's list of the (step, lane) lookups, to be shared out over
         //     the lanes so that their loads overlap (a3) ---------------------------
-        const bool grid = (FX || !p.constant_mode) && p.occ;
+        const bool grid = (VOL != kAnyVolume || !p.constant_mode) && p.occ;
         uint32_t need = 0;
         unsigned nq = 0;
         const auto list = [&](int k, bool nd) {
@@ -594,7 +618,7 @@ __device__ __forceinline__ unsigned march_tile(
                     bool o[kScan];
 #pragma unroll
                     for (int k = 0; k < kScan; ++k) {
-                        o[k] = occupied<FX>(p, bx, by, bz);
+                        o[k] = occupied<VOL>(p, bx, by, bz);
                         bx = mad32(d.x, p.one, bx);
                         by = mad32(d.y, p.one, by);
                         bz = mad32(d.z, p.one, bz);
@@ -627,7 +651,7 @@ __device__ __forceinline__ unsigned march_tile(
                 uint32_t bx = s.x + i0 * d.x, by = s.y + i0 * d.y, bz = s.z + i0 * d.z;
 #pragma unroll
                 for (int k = 0; k < CH; ++k) {
-                    o[k] = occupied<FX>(p, bx, by, bz);
+                    o[k] = occupied<VOL>(p, bx, by, bz);
                     bx = mad32(d.x, p.one, bx);
                     by = mad32(d.y, p.one, by);
                     bz = mad32(d.z, p.one, bz);
@@ -663,7 +687,7 @@ __device__ __forceinline__ unsigned march_tile(
             for (int b = 0; b < kViewBatch; ++b) {
                 uint32_t cs[kLatticeAxes];
                 const int32_t hs = step_coords(p, ws, pr[b] & 31u, (uint32_t)i0 + (pr[b] >> 5), cs);
-                rho[b] = density<FX>(p, base, detail, weather, cs, hs).value();
+                rho[b] = density<VOL>(p, base, detail, weather, cs, hs).value();
             }
 #pragma unroll
             for (int b = 0; b < kViewBatch; ++b) ws.rho[pr[b] >> 5][pr[b] & 31u] = rho[b];
@@ -720,14 +744,14 @@ __device__ __forceinline__ unsigned march_tile(
             // every lane are left out (their density is 0)
             const int32_t h_least = __reduce_min_sync(kFull, hs);
             int nl = nlight;
-            while (nl > 0 && h_least + p.lh[nl - 1] >= p.h_top && (FX || !p.constant_mode)) --nl;
+            while (nl > 0 && h_least + p.lh[nl - 1] >= p.h_top && (VOL != kAnyVolume || !p.constant_mode)) --nl;
             float rho_sum = 0.0f;
-            constexpr int kU = LightUnroll<T, FX>::value;
+            constexpr int kU = LightUnroll<T, VOL>::value;
 #pragma unroll kU
             for (int j = 0; j < nl; ++j) {
                 uint32_t cj[kLatticeAxes];
-                light_coords<FX>(p, cs, j, cj);
-                const Density d = density<FX>(p, base, detail, weather, cj, hs + p.lh[j]);
+                light_coords<VOL>(p, cs, j, cj);
+                const Density d = density<VOL>(p, base, detail, weather, cj, hs + p.lh[j]);
                 rho_sum = fmaf(d.gw, d.r, rho_sum);
             }
             if (!ok) continue;
@@ -791,10 +815,10 @@ void launch_march_ch(const SceneParams &p, const ViewParams &v, const cloud_volu
 void launch_march_small(const SceneParams &p, const ViewParams &v, const cloud_volume *vol,
                         unsigned long long *counter, int shape, cudaStream_t s);
 template <int CH>
-const void *batch_kernel_ch(int precision, int light_steps, bool fx, int shape);
-// True when a launch can use the FX march: the standard tile sizes, all three
-// tiles present, noise density, six light steps and a base tile period of 2^k
-// detail periods (the detail coordinates then follow from the base ones).
-bool fixed_sizes(const SceneParams &p, const cloud_volume *vol);
+const void *batch_kernel_ch(int precision, int kind, int shape);
+// The kind of march a launch takes: standard needs the standard tile sizes, all
+// three tiles and a base tile period of 2^k detail periods (the detail coordinates
+// then follow from the base ones); base neither a detail nor a weather tile.
+int volume_kind(const SceneParams &p, const cloud_volume *vol);
 
 }  // namespace cloudvol

@@ -3,5 +3,5 @@
 #include "march_kernels.cuh"
 
 namespace cloudvol {
-template const void *batch_kernel_ch<8>(int, int, bool, int);
+template const void *batch_kernel_ch<8>(int, int, int);
 }  // namespace cloudvol

@@ -1,6 +1,5 @@
 // march_kernels.cuh -- the raymarch kernels (one view; many views from a work
-// queue) and their dispatch over storage type, light-step specialisation, tile
-// sizes and tile shape, for one chunk size CH.  Included only by
+// queue) and their dispatch over storage type, kind of volume and tile shape, for one chunk size CH.  Included only by
 // march{8,16}_{view,batch}.cu, which instantiate the single-view and the
 // multi-view kernels for CH = 8 and CH = 16 (four units compiled in parallel).
 #pragma once
@@ -9,13 +8,13 @@
 
 namespace cloudvol {
 
-template <typename T, int LS, int SHAPE, bool FX, int CH, int STEPS>
-__global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
+template <typename T, int SHAPE, int VOL, int CH, int STEPS>
+__global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH>::value)
     march_kernel(const __grid_constant__ SceneParams p, const __grid_constant__ ViewParams v,
                  const T *__restrict__ base, const T *__restrict__ detail,
                  const T *__restrict__ weather, unsigned long long *__restrict__ counter) {
-    __shared__ WarpScratch<CH, FX> scratch[4];
-    const unsigned n = march_tile<T, LS, SHAPE, FX, CH, STEPS>(
+    __shared__ WarpScratch<CH, VOL> scratch[4];
+    const unsigned n = march_tile<T, SHAPE, VOL, CH, STEPS>(
         p, v, blockIdx.x, blockIdx.y, scratch[threadIdx.x >> 5], base, detail, weather);
     count_lookups(counter, n);
 }
@@ -24,13 +23,13 @@ __global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
 // items from a device counter until the queue is empty; the view of an item
 // is found by binary search over the views' first tile indices and staged in
 // shared memory.
-template <typename T, int LS, int SHAPE, bool FX, int CH>
-__global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
+template <typename T, int SHAPE, int VOL, int CH>
+__global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH>::value)
     march_batch_kernel(const __grid_constant__ SceneParams p, const ViewParams *__restrict__ views,
                        int n_views, int total_tiles, unsigned int *__restrict__ work,
                        const T *__restrict__ base, const T *__restrict__ detail,
                        const T *__restrict__ weather, unsigned long long *__restrict__ counter) {
-    __shared__ WarpScratch<CH, FX> scratch[4];
+    __shared__ WarpScratch<CH, VOL> scratch[4];
     __shared__ ViewParams sv;
     __shared__ int s_tile, s_view;
     unsigned long long n_look = 0;
@@ -57,7 +56,7 @@ __global__ void __launch_bounds__(128, MarchBlocks<T, FX, CH>::value)
         __syncthreads();
         const int local = t - sv.tile_begin;
         if (in_range(p.check, s_view >= 0 && s_view < n_views && local >= 0 && t < total_tiles, kChkView))
-            n_look += march_tile<T, LS, SHAPE, FX, CH, kAnySteps>(p, sv, local % sv.tiles_x, local / sv.tiles_x,
+            n_look += march_tile<T, SHAPE, VOL, CH, kAnySteps>(p, sv, local % sv.tiles_x, local / sv.tiles_x,
                                                        scratch[threadIdx.x >> 5], base, detail, weather);
         __syncthreads();  // s_tile / sv are rewritten by the next iteration
     }
@@ -71,13 +70,18 @@ void launch_shape(const SceneParams &p, const ViewParams &v, const cloud_volume 
     tile_dims(SHAPE, &tw, &th);
     const dim3 grid(v.tiles_x, (v.height + th - 1) / th);
     const T *b = (const T *)vol->base, *d = (const T *)vol->detail, *w = (const T *)vol->weather;
-    if (fixed_sizes(p, vol))
-        if (v.steps <= CH) march_kernel<T, 6, SHAPE, true, CH, kOneChunk><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
-        else march_kernel<T, 6, SHAPE, true, CH, kManyChunks><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
-    else if (p.light_steps == 6)
-        march_kernel<T, 6, SHAPE, false, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
-    else
-        march_kernel<T, -1, SHAPE, false, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+    switch (volume_kind(p, vol)) {
+        case kStandardVolume:
+            if (v.steps <= CH)
+                march_kernel<T, SHAPE, kStandardVolume, CH, kOneChunk><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+            else
+                march_kernel<T, SHAPE, kStandardVolume, CH, kManyChunks><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+            break;
+        case kBaseVolume:
+            march_kernel<T, SHAPE, kBaseVolume, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+            break;
+        default: march_kernel<T, SHAPE, kAnyVolume, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
+    }
 }
 
 template <typename T, int CH>
@@ -103,27 +107,29 @@ void launch_march_ch(const SceneParams &p, const ViewParams &v, const cloud_volu
 }
 
 template <typename T, int SHAPE, int CH>
-const void *batch_kernel_ptr(int light_steps, bool fx) {
-    if (fx) return (const void *)march_batch_kernel<T, 6, SHAPE, true, CH>;
-    return light_steps == 6 ? (const void *)march_batch_kernel<T, 6, SHAPE, false, CH>
-                            : (const void *)march_batch_kernel<T, -1, SHAPE, false, CH>;
+const void *batch_kernel_ptr(int kind) {
+    switch (kind) {
+        case kStandardVolume: return (const void *)march_batch_kernel<T, SHAPE, kStandardVolume, CH>;
+        case kBaseVolume: return (const void *)march_batch_kernel<T, SHAPE, kBaseVolume, CH>;
+        default: return (const void *)march_batch_kernel<T, SHAPE, kAnyVolume, CH>;
+    }
 }
 template <typename T, int CH>
-const void *batch_kernel_typed(int light_steps, bool fx, int shape) {
+const void *batch_kernel_typed(int kind, int shape) {
     switch (shape) {
-        case 1: return batch_kernel_ptr<T, 1, CH>(light_steps, fx);
-        case 2: return batch_kernel_ptr<T, 2, CH>(light_steps, fx);
-        case 3: return batch_kernel_ptr<T, 3, CH>(light_steps, fx);
-        default: return batch_kernel_ptr<T, 0, CH>(light_steps, fx);
+        case 1: return batch_kernel_ptr<T, 1, CH>(kind);
+        case 2: return batch_kernel_ptr<T, 2, CH>(kind);
+        case 3: return batch_kernel_ptr<T, 3, CH>(kind);
+        default: return batch_kernel_ptr<T, 0, CH>(kind);
     }
 }
 template <int CH>
-const void *batch_kernel_ch(int precision, int light_steps, bool fx, int shape) {
+const void *batch_kernel_ch(int precision, int kind, int shape) {
     switch (precision) {
-        case CLOUD_PRECISION_FP32: return batch_kernel_typed<float, CH>(light_steps, fx, shape);
-        case CLOUD_PRECISION_FP16: return batch_kernel_typed<__half, CH>(light_steps, fx, shape);
-        case CLOUD_PRECISION_BF16: return batch_kernel_typed<__nv_bfloat16, CH>(light_steps, fx, shape);
-        default: return batch_kernel_typed<uint16_t, CH>(light_steps, fx, shape);
+        case CLOUD_PRECISION_FP32: return batch_kernel_typed<float, CH>(kind, shape);
+        case CLOUD_PRECISION_FP16: return batch_kernel_typed<__half, CH>(kind, shape);
+        case CLOUD_PRECISION_BF16: return batch_kernel_typed<__nv_bfloat16, CH>(kind, shape);
+        default: return batch_kernel_typed<uint16_t, CH>(kind, shape);
     }
 }
 

@@ -223,10 +223,13 @@ static int small_shape(int width, int height) {
     return pixels <= 2 * wave ? 6 : pixels <= 8 * wave ? 5 : pixels <= 16 * wave ? 4 : -1;
 }
 
-bool fixed_sizes(const SceneParams &p, const cloud_volume *vol) {
-    return p.light_steps == 6 && !p.constant_mode && vol->detail && vol->weather &&
-           p.log2_base == kStdLog2Base && p.log2_detail == kStdLog2Detail &&
-           p.log2_weather == kStdLog2Weather && p.detail_shift >= 0;
+int volume_kind(const SceneParams &p, const cloud_volume *vol) {
+    if (p.constant_mode) return kAnyVolume;
+    if (!vol->detail && !vol->weather) return kBaseVolume;
+    return vol->detail && vol->weather && p.log2_base == kStdLog2Base && p.log2_detail == kStdLog2Detail &&
+                   p.log2_weather == kStdLog2Weather && p.detail_shift >= 0
+               ? kStandardVolume
+               : kAnyVolume;
 }
 
 int launch_march(const SceneParams &p, const ViewParams &v, const cloud_volume *vol,

@@ -78,12 +78,13 @@ def test_partial_and_clear_chunks(api, oracle, steps, config):
 # 9728, 38912 and 77824 pixels, ragged against every tile; the multi-view launch always has 32
 @pytest.mark.parametrize("w,h", [(1, 1), (5, 3), (64, 152), (97, 101), (256, 152), (261, 151), (304, 256),
                                  (307, 257)])
-@pytest.mark.parametrize("kind,precision", [("full", "fp32"), ("full", "bf16"), ("tiny", "fp32"),
-                                            ("tiny", "unorm16")])
+@pytest.mark.parametrize("kind,precision,base_n", [("full", "fp32", 128), ("full", "bf16", 128),
+                                                   ("full", "fp16", 64), ("tiny", "fp32", 64),
+                                                   ("tiny", "unorm16", 32)])
 @pytest.mark.parametrize("steps", [8, 21])
-def test_small_images_equal_batched_views(api, w, h, kind, precision, steps):
+def test_small_images_equal_batched_views(api, w, h, kind, precision, base_n, steps):
     import torch
-    vol = api.Volume(I.volume_desc(kind, seed=8, precision=precision))
+    vol = api.Volume(I.volume_desc(kind, seed=8, precision=precision, base_n=base_n))
     cam = I.camera((100.0, -700.0, 500.0), 210.0, 36.0, 60.0)
     view = dict(camera=cam, width=w, height=h, steps=steps, jitter_frame=5)
     for light_steps in (6, 3):
