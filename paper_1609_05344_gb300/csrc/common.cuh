@@ -98,6 +98,7 @@ struct cloud_volume {
     // occupancy grid: one bit per cell of 2^kOccShift base records per axis (x fastest),
     // clear where the density is provably 0 throughout (see build_occupancy)
     uint32_t *occ;   // device or nullptr (constant density)
+    uint32_t *occ_blocks;  // the same bits in blocks of 16^3 cells, or nullptr (not 256^3 cells)
     int log2_occ;    // macro-cells per axis = 2^log2_occ = base_n / 2^kOccShift
     int device;
 };

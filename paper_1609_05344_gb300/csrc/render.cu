@@ -87,6 +87,7 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
     p->inv_1mc = (float)(1.0 / (1.0 - d.coverage));
     p->rho0 = (float)d.constant_density;
     p->occ = noise && g_use_occupancy.load() ? vol->occ : nullptr;
+    p->occ_blocks = p->occ ? vol->occ_blocks : nullptr;
     p->log2_occ = vol->log2_occ;
     p->check = check_word();
     p->log2_base = vol->log2_base;

@@ -402,6 +402,22 @@ __global__ void occupancy_half_kernel(const T *__restrict__ base, int log2b,
     }
 }
 
+// The 256^3 grid copied into blocks of 16^3 cells: cell (X, Y, Z) is bit
+// [Z hi, Y hi, X hi, Z lo, Y lo, X lo] (nibbles, highest first).
+__global__ void occupancy_blocks_kernel(const uint32_t *__restrict__ occ, uint32_t *__restrict__ blocks) {
+    const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= 1u << 19) return;
+    uint32_t bits = 0;
+    for (uint32_t b = 0; b < 32; ++b) {
+        const uint32_t i = 32 * w + b;
+        const uint32_t x = (i & 15u) | ((i >> 8) & 0xF0u), y = ((i >> 4) & 15u) | ((i >> 12) & 0xF0u),
+                       z = ((i >> 8) & 15u) | ((i >> 16) & 0xF0u);
+        const uint32_t cell = (z << 16) | (y << 8) | x;
+        bits |= ((occ[cell >> 5] >> (cell & 31u)) & 1u) << b;
+    }
+    blocks[w] = bits;
+}
+
 // Extremes of the corners of every record of a tile (for occupancy bounds
 // that cannot localise the detail tile); one block of 1024 threads.
 template <typename T>
@@ -486,7 +502,12 @@ int build_occupancy(cloud_volume *v, cudaStream_t s) {
         occupancy_kernel<T><<<grid_for(words, 128), 128, 0, s>>>(
             (const T *)v->base, v->log2_base, (const T *)v->detail, v->log2_detail, (float)ratio, range[0],
             range[1], k0, (float)wd, v->occ);
-    return check_launch("occupancy_kernel");
+    if (int rc = check_launch("occupancy_kernel")) return rc;
+    if (v->log2_occ != 8) return CLOUD_OK;
+    if (int rc = check_cuda(cudaMalloc(&v->occ_blocks, words * sizeof(uint32_t)), "cudaMalloc occupancy blocks"))
+        return rc;
+    occupancy_blocks_kernel<<<(unsigned)(words / 256), 256, 0, s>>>(v->occ, v->occ_blocks);
+    return check_launch("occupancy_blocks_kernel");
 }
 
 // Generates each tile in FP64 into a plain scratch array, corner-packs it into
@@ -548,6 +569,7 @@ void free_volume(cloud_volume *v) {
     if (v->detail) cudaFree(v->detail);
     if (v->weather) cudaFree(v->weather);
     if (v->occ) cudaFree(v->occ);
+    if (v->occ_blocks) cudaFree(v->occ_blocks);
     delete v;
 }
 
