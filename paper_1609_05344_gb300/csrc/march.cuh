@@ -31,12 +31,12 @@
 
 namespace cloudvol {
 
-// Records at the standard tile sizes, 8 view steps per warp iteration: 8 CTAs
-// (64 registers, no spills; FP32 148.8 us at fast-1080p against 154.5 us with
-// 7 and 154.2 us with 9; FP16 152.4 us against 153.0 us with 7).  With 16 steps
-// per iteration the per-warp scratch is 1.7x larger and 8 CTAs would leave the
-// L1 28 KB: 7 CTAs for FP32 records and 6 for 16-bit ones (the 64-view batch,
-// BF16: 18.7 ms against 19.5 ms with 8).
+// Records at the standard tile sizes and base tiles alone, 8 view steps per warp
+// iteration: 8 CTAs (64 registers, no spills; 1920x1080 x 8 steps, FP32: 83.4 us,
+// 83.3 with 7, 84.3 with 6, 86.5 with 9; 64 views, BF16: 10.50 ms, 10.73 with 7,
+// 10.96 with 6).  With 16 steps per iteration the per-warp scratch is 1.7x larger
+// and 8 CTAs would leave the L1 28 KB: 7 CTAs for FP32 records and 6 for 16-bit
+// ones (64 views, BF16, by an earlier build: 18.7 ms against 19.5 ms with 8).
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX
 #define CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX 8
 #endif
@@ -467,12 +467,15 @@ __device__ __forceinline__ float step_depth(float absorption, float rho, float D
 //      weight), which phase C would evaluate with only the lanes busy that have
 //      density at that step;
 //   C  each lane sums its steps in order.
-// What bounds it is instruction issue together with the latency of the lookups,
-// so work moves to where most lanes are busy.  With the exponentials in phase B,
-// the list of light marches compacted from the list of lookups (instead of
-// listed anew), rays staged in 16-byte groups and clear chunks left at once,
-// the 1920x1080 8-step frame takes 95.0 us (112.5 before), 1280x720 with 128
-// steps 430 us (538), 64 uneven views 12.58 ms (15.21); the same pixels bitwise.
+// What bounds it is the L1's data path (83 % busy) where every ray has an offset
+// of its own, and instruction issue (75 %) with the latency of the lookups
+// elsewhere, so work moves to where most lanes are busy.  The exponentials in
+// phase B, the list of light marches compacted from the list of lookups (instead of
+// listed anew), rays staged in 16-byte groups and clear chunks left at once took
+// 1920x1080 x 8 steps from 112.5 to 95.0 us, 1280x720 x 128 steps from 538 to 430
+// us and 64 uneven views from 15.21 to 12.58 ms; with the steps described at the
+// parts below, 128.7 to 91.4 us, 565 to 370 us and 15.5 to 10.2 ms a pass (other
+// cameras).
 // The arithmetic of every sample is the same as a per-lane march (a skipped
 // lookup is one whose density is exactly 0).  Returns the number of density
 // lookups this lane's ray performed in the method's sense (Sec. 1: one per

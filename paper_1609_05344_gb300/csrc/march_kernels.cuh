@@ -1,7 +1,8 @@
 // march_kernels.cuh -- the raymarch kernels (one view; many views from a work
-// queue) and their dispatch over storage type, kind of volume and tile shape, for one chunk size CH.  Included only by
-// march{8,16}_{view,batch}.cu, which instantiate the single-view and the
-// multi-view kernels for CH = 8 and CH = 16 (four units compiled in parallel).
+// queue) and their dispatch over storage type, kind of volume and tile shape, for
+// one chunk size CH.  Included only by march{8,16}_{view,batch}.cu, which
+// instantiate the single-view and the multi-view kernels for CH = 8 and CH = 16,
+// and march_small.cu (five units compiled in parallel).
 #pragma once
 
 #include "march.cuh"

@@ -1,11 +1,11 @@
 // render.cu -- single-view raymarch launch (cloud_render) and the host-side
 // construction of the launch constants (Sec. 1, Sec. 3.1, Sec. 3.2).
 //
-// One thread per pixel; a 128-thread CTA covers one pixel tile (shape chosen
-// by the autotuner, 16x8 by default) so the rays of a warp stay adjacent and
-// touch the same region of the L2-resident noise tiles.  The device code is
-// in march.cuh, the kernels in march_kernels.cuh (instantiated by
-// march{8,16}_{view,batch}.cu).
+// One lane per pixel; a 128-thread CTA covers one pixel tile (shape chosen by the
+// autotuner, 8x16 by default, smaller ones with idle lanes for small images) so the
+// rays of a warp stay adjacent and touch the same region of the L2-resident noise
+// tiles.  The device code is in march.cuh, the kernels in march_kernels.cuh
+// (instantiated by march{8,16}_{view,batch}.cu and march_small.cu).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -188,8 +188,8 @@ int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_cam
 
 // ---------------------------------------------------------------------------
 // Launch-configuration selection: the autotuner records the fastest (tile
-// shape, view steps per warp iteration) per (storage precision, light-step
-// specialisation); launches use it when present.
+// shape, view steps per warp iteration) per (storage precision, six light steps
+// or another number); launches use it when present.
 namespace {
 std::mutex g_tune_mu;
 int g_best_config[4][2] = {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}};

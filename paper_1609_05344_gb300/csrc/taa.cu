@@ -243,7 +243,7 @@ __device__ __forceinline__ float4 blend4(float4 h, float4 c, float b) {
 // ResolvePix<H> vertically adjacent pixels, whose 3x3 windows share rows, and
 // filters their history footprints before it waits for the tile.
 #ifndef CLOUDVOL_TAA_PIX_F32
-#define CLOUDVOL_TAA_PIX_F32 4  // pixels per thread, FP32 history (79 registers)
+#define CLOUDVOL_TAA_PIX_F32 4  // pixels per thread, FP32 history (78 registers)
 #endif
 #ifndef CLOUDVOL_TAA_PIX_F16
 #define CLOUDVOL_TAA_PIX_F16 2  // pixels per thread, FP16 history
