@@ -204,12 +204,13 @@ struct TileShape<5> { static constexpr int WX = 4, WY = 2, CX = 2, CY = 2; };
 template <>
 struct TileShape<6> { static constexpr int WX = 2, WY = 2, CX = 2, CY = 2; };
 inline void tile_dims(int shape, int *tw, int *th) {
-    static const int w[kAllShapes] = {16, 32, 32, 8, 8, 8, 4}, h[kAllShapes] = {8, 4, 4, 16, 8, 4, 4};
+    // not static: a static local of an inline function is one object per process,
+    // also between two builds of the library
+    constexpr int w[kAllShapes] = {16, 32, 32, 8, 8, 8, 4}, h[kAllShapes] = {8, 4, 4, 16, 8, 4, 4};
     *tw = w[shape];
     *th = h[shape];
 }
 
-constexpr int kAxes = kLatticeAxes + 1;  // lattice axes + height above the layer bottom
 // Launch configurations the autotuner chooses from: a pixel-tile shape and the
 // number of view steps a warp evaluates per iteration of its march (the chunk
 // of phase A/B/C below).  config = shape + kShapes * chunk index.
