@@ -49,13 +49,14 @@ namespace cloudvol {
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16
 #define CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16 6
 #endif
-// What a march is compiled for: any volume; the standard tile sizes (below); a
-// base tile of any size alone, with neither detail nor weather, which needs a
-// third of the records and registers for 8 CTAs (64^3 base, 1280x720 x 64 steps
-// 520.7 us as any volume, 307.5 as this).  The number of light steps is a launch
+// What a march is compiled for: any volume of noise tiles; the standard tile sizes
+// (below); a base tile of any size alone, with neither detail nor weather, which
+// needs a third of the records and registers for 8 CTAs (64^3 base, 1280x720 x 64
+// steps 520.7 us as any volume, 307.5 as this); constant density (FP32 kernels
+// only: it has no records).  The number of light steps is a launch
 // value: compiled in, it gained nothing, and kept standard volumes with other
 // than six light steps (nine: 480 -> 431 us) from their own kernel.
-enum VolumeKind { kAnyVolume, kStandardVolume, kBaseVolume };
+enum VolumeKind { kAnyVolume, kStandardVolume, kBaseVolume, kConstantVolume };
 template <typename T, int VOL, int CH>
 struct MarchBlocks {
     static constexpr bool f32 = sizeof(T) == 4;
@@ -136,7 +137,7 @@ struct SceneParams {
     int log2_occ;
     unsigned *check;  // status word of the checked build, else nullptr
     int log2_base, log2_detail, log2_weather;
-    int light_steps, integration, constant_mode;
+    int light_steps, integration;
     int wide;  // t_max spans more than 1000 tile periods (df_to_u32)
     // detail coordinates = base detail_mul + detail_add (mod 2^32) when the base
     // tile period is 2^detail_shift detail periods (-1: convert separately)
@@ -363,7 +364,6 @@ __device__ __forceinline__ Density density(const SceneParams &p, const T *__rest
     const bool has_detail = FX || (VOL == kAnyVolume && detail), has_weather = FX || (VOL == kAnyVolume && weather);
     const int lb = FX ? kStdLog2Base : p.log2_base, ld = FX ? kStdLog2Detail : p.log2_detail,
               lw = FX ? kStdLog2Weather : p.log2_weather;
-    if (VOL == kAnyVolume && p.constant_mode) return {p.rho0, 1.0f};
     const float g = height_profile(p, hq);
     float cb[8], cd[8], cw[4];
     const uint32_t rb = rec3(p.base_mul, lb, c[kBX], c[kBY], c[kBZ]),
@@ -452,6 +452,14 @@ __device__ __forceinline__ int32_t step_coords(const SceneParams &p, const WarpS
 // sigma D of one step, rounded the same way wherever it is recomputed
 __device__ __forceinline__ float step_depth(float absorption, float rho, float D) {
     return __fmul_rn(__fmul_rn(absorption, rho), D);
+}
+// Weight of a step of depth sd behind the optical depth t0 (a6, Sec. 3.1).
+__device__ __forceinline__ float step_weight(const SceneParams &p, float t0, float sd) {
+    return p.integration == CLOUD_INTEGRATE_ANALYTIC ? expf(-t0) * -expm1f(-sd) : expf(-__fadd_rn(t0, sd)) * sd;
+}
+// Transmittance towards the sun of a light march's density sum (a5).
+__device__ __forceinline__ float sun_transmittance(const SceneParams &p, float rho_sum) {
+    return expf(-p.absorption * p.light_step * rho_sum);
 }
 
 // The march of one CTA pixel tile (4 warps, one pixel per lane).  View steps
@@ -570,7 +578,7 @@ __device__ __forceinline__ unsigned march_tile(
             for (int k = 0; k < 3; ++k) pos[k] = df2_mul_raw(ld, {both(r[k].hi), both(r[k].lo)});
             const bool wide = p.wide != 0;
 #pragma unroll
-            for (int a = 0; a < kLatticeAxes; ++a) {
+            for (int a = 0; VOL != kConstantVolume && a < kLatticeAxes; ++a) {
                 if (a >= kDX && a <= kDZ && p.detail_shift >= 0) {
                     // same origin, period 2^-shift of the base tile: exact shift
                     c[a] = mad32(c[a - kDX], p.detail_mul, p.detail_add);
@@ -598,15 +606,42 @@ __device__ __forceinline__ unsigned march_tile(
             phase = p.hg_norm * q * q * q;
         }
     }
-    stage_ray(ws, lane, c, e, hq, eh);
-    ws.length[lane] = Df;
-    __syncwarp();
+    if (VOL != kConstantVolume) {
+        stage_ray(ws, lane, c, e, hq, eh);
+        ws.length[lane] = Df;
+        __syncwarp();
+    }
     const unsigned lt_mask = (1u << lane) - 1u;
     float tau = 0.0f, cr = 0.0f, cg = 0.0f, cb = 0.0f;
+    if (VOL == kConstantVolume && alive) {
+        // Constant density: nothing to look up and the same light march at every step,
+        // so each lane walks its own steps (one exponential a step bounds it).  The
+        // lists below pay only where lanes lack work: through them, 1280x720 x 64 steps
+        // take 370 us (283 with the light samples unrolled), this way 24.6; 12 views of
+        // up to 1280x720 x 128 steps 2.59 ms and 0.24.
+        float rho_sum = 0.0f;
+        for (int j = 0; j < nlight; ++j) rho_sum = __fadd_rn(rho_sum, p.rho0);
+        const float sd = step_depth(p.absorption, p.rho0, Df), sun_t = sun_transmittance(p, rho_sum) * phase;
+        const float lr = fmaf(p.sun_rad[0], sun_t, p.ambient[0]), lg = fmaf(p.sun_rad[1], sun_t, p.ambient[1]),
+                    lb = fmaf(p.sun_rad[2], sun_t, p.ambient[2]);
+        int i = 0;
+        do {
+            ++i;
+            if (p.rho0 > 0.0f) {
+                const float wgt = step_weight(p, tau, sd);
+                tau = __fadd_rn(tau, sd);
+                cr = fmaf(wgt, lr, cr);
+                cg = fmaf(wgt, lg, cg);
+                cb = fmaf(wgt, lb, cb);
+            }
+        } while (i < v.steps && !(tau >= p.tau_max));
+        n_look = i * (p.rho0 > 0.0f ? 1 + nlight : 1);
+    }
     constexpr int kScan = 16;  // steps per read of the grid in a march of many chunks
     uint32_t occ_bits = 0;
     int scanned = 0;
-    for (int i0 = 0; i0 < (STEPS == kOneChunk ? 1 : v.steps) && __any_sync(kFull, alive); i0 += CH) {
+    for (int i0 = 0; VOL != kConstantVolume && i0 < (STEPS == kOneChunk ? 1 : v.steps) && __any_sync(kFull, alive);
+         i0 += CH) {
         const int nst = min(CH, v.steps - i0);
         // --- A1: which of this lane's CH steps need a density lookup: those in an
         //     occupied macro-cell of the occupancy grid (the words of all steps are
@@ -616,7 +651,7 @@ __device__ __forceinline__ unsigned march_tile(
         //     left to the lookup.
         // --- A2: the warp's list of the (step, lane) lookups, to be shared out over
         //     the lanes so that their loads overlap (a3) ---------------------------
-        const bool grid = (VOL != kAnyVolume || !p.constant_mode) && p.occ;
+        const bool grid = p.occ;
         uint32_t need = 0;
         unsigned nq = 0;
         const auto list = [&](int k, bool nd) {
@@ -772,7 +807,7 @@ __device__ __forceinline__ unsigned march_tile(
             // every lane are left out (their density is 0)
             const int32_t h_least = __reduce_min_sync(kFull, hs);
             int nl = nlight;
-            while (nl > 0 && h_least + p.lh[nl - 1] >= p.h_top && (VOL != kAnyVolume || !p.constant_mode)) --nl;
+            while (nl > 0 && h_least + p.lh[nl - 1] >= p.h_top) --nl;
             // A lane without a pair leaves here with FP32 records, whose 80 bytes a
             // lane and sample fill the L1's data path (1920x1080 x 8 steps 115.0 ->
             // 112.0 us, 1280x720 x 128 steps 485 -> 477 us); with 16-bit ones it
@@ -793,10 +828,8 @@ __device__ __forceinline__ unsigned march_tile(
             //     per-step integral (Sec. 3.1) --------------------------------
             const float sd = step_depth(p.absorption, ws.rho[k][ow], ws.length[ow]);
             const float t0 = ws.aux[k][ow];
-            ws.rho[k][ow] = p.integration == CLOUD_INTEGRATE_ANALYTIC
-                                ? expf(-t0) * -expm1f(-sd)
-                                : expf(-__fadd_rn(t0, sd)) * sd;
-            ws.aux[k][ow] = expf(-p.absorption * p.light_step * rho_sum);
+            ws.rho[k][ow] = step_weight(p, t0, sd);
+            ws.aux[k][ow] = sun_transmittance(p, rho_sum);
         }
         __syncwarp();
         // --- C: in-scattered light, summed in step order -------------------------
@@ -852,7 +885,8 @@ template <int CH>
 const void *batch_kernel_ch(int precision, int kind, int shape);
 // The kind of march a launch takes: standard needs the standard tile sizes, all
 // three tiles and a base tile period of 2^k detail periods (the detail coordinates
-// then follow from the base ones); base neither a detail nor a weather tile.
+// then follow from the base ones); base neither a detail nor a weather tile;
+// constant no tile at all.
 int volume_kind(const SceneParams &p, const cloud_volume *vol);
 
 }  // namespace cloudvol

@@ -81,6 +81,10 @@ void launch_shape(const SceneParams &p, const ViewParams &v, const cloud_volume 
         case kBaseVolume:
             march_kernel<T, SHAPE, kBaseVolume, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
             break;
+        case kConstantVolume:
+            march_kernel<float, SHAPE, kConstantVolume, CH, kAnySteps>
+                <<<grid, 128, 0, s>>>(p, v, nullptr, nullptr, nullptr, counter);
+            break;
         default: march_kernel<T, SHAPE, kAnyVolume, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
     }
 }
@@ -112,6 +116,7 @@ const void *batch_kernel_ptr(int kind) {
     switch (kind) {
         case kStandardVolume: return (const void *)march_batch_kernel<T, SHAPE, kStandardVolume, CH>;
         case kBaseVolume: return (const void *)march_batch_kernel<T, SHAPE, kBaseVolume, CH>;
+        case kConstantVolume: return (const void *)march_batch_kernel<float, SHAPE, kConstantVolume, CH>;
         default: return (const void *)march_batch_kernel<T, SHAPE, kAnyVolume, CH>;
     }
 }

@@ -95,7 +95,6 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
     p->log2_weather = vol->log2_weather;
     p->light_steps = light_steps;
     p->integration = integration;
-    p->constant_mode = noise ? 0 : 1;
     double least_period = d.base_period_m;
     if (noise && vol->log2_detail) least_period = std::min(least_period, d.detail_period_m);
     if (noise && vol->log2_weather) least_period = std::min(least_period, d.weather_period_m);
@@ -225,7 +224,7 @@ static int small_shape(int width, int height) {
 }
 
 int volume_kind(const SceneParams &p, const cloud_volume *vol) {
-    if (p.constant_mode) return kAnyVolume;
+    if (vol->desc.density_mode != CLOUD_DENSITY_NOISE) return kConstantVolume;
     if (!vol->detail && !vol->weather) return kBaseVolume;
     return vol->detail && vol->weather && p.log2_base == kStdLog2Base && p.log2_detail == kStdLog2Detail &&
                    p.log2_weather == kStdLog2Weather && p.detail_shift >= 0

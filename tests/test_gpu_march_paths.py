@@ -92,3 +92,24 @@ def test_small_images_equal_batched_views(api, w, h, kind, precision, base_n, st
         batch = api.Batch(vol, I.params(), [view], light_steps)
         assert torch.equal(one, batch.render()[0])
         assert int(count.item()) >= int((one[..., 3] > 0).sum().item())
+
+
+# constant density: both rules, no, one and the most light steps, the early out after a few
+# steps, at once, never and off, no density at all; below, inside and above the layer
+@pytest.mark.parametrize("rho0,tau_max", [(0.05, 11.5), (0.002, 0.7), (0.05, 1e-6), (1e-5, 0.0), (0.0, 11.5)])
+@pytest.mark.parametrize("integration,light_steps", [("analytic", 6), ("basic", 1), ("analytic", 0), ("basic", 32)])
+@pytest.mark.parametrize("height,pitch,w,h,steps", [(500.0, 20.0, 45, 31, 9), (2500.0, 0.0, 307, 257, 21),
+                                                    (5200.0, -30.0, 1, 1, 130)])
+def test_constant_density(api, oracle, rho0, tau_max, integration, light_steps, height, pitch, w, h, steps):
+    desc, prm = I.volume_desc("constant", rho0=rho0), I.params(tau_max=tau_max)
+    cam = I.camera((0.0, 0.0, height), 70.0, pitch, 60.0)
+    vol, ovol = api.Volume(desc), oracle.Volume(desc)
+    got, count = api.render(vol, cam, prm, w, h, steps, light_steps, jitter_frame=4, integration=integration,
+                            count=True)
+    rule = oracle.ANALYTIC if integration == "analytic" else oracle.BASIC
+    ref, n = oracle.render(ovol, cam, prm, w, h, steps, light_steps, jitter_frame=4, integration=rule, nthreads=8)
+    assert np.abs(got.cpu().numpy() - ref).max() <= TOL["fp32"]
+    assert abs(int(count.item()) - n) <= 1e-3 * n + (0 if rho0 == 0.0 else 1 + light_steps)
+    view = dict(camera=cam, width=w, height=h, steps=steps, jitter_frame=4)
+    batch = api.Batch(vol, prm, [view, view], light_steps, integration)
+    assert all(np.array_equal(o.cpu().numpy(), got.cpu().numpy()) for o in batch.render())
