@@ -18,23 +18,32 @@
 
 #include "common.cuh"
 
-// CTAs per SM the march is compiled for (register budget 65536 / (128 x this)),
-// for FP32 records and for 16-bit records (which need fewer registers): volumes of
-// any tile sizes (64^3 base, 1280x720 x 64 steps: 234.4 us against 242.6 with 5;
-// FP16 236.7 against 243.7 with 6).
+// CTAs per SM the march of volumes of any tile sizes is compiled for (register budget
+// 65536 / (128 x this)).  FP32 records: six for one view, five for the multi-view
+// kernel, whose loop needs more registers; 16-bit records: six for both.  More of them
+// spill, and cost more than the occupancy gives (64^3 base with detail and weather).
+// FP16, six against seven (80 against 72 registers): 307x257 x 64 steps 74.5 us against
+// 84.1, 12 views of 8 to 128 steps 1.27 ms against 1.33, 16 small ones 52 us against 63.
+// FP32, one view, six against five: 256x152 x 8 steps (detail at 700 m) 10.4 us against
+// 12.2, 1280x720 x 64 steps 227 us against 231; many views, five against six: 16 small
+// ones 46 us against 51, 12 larger ones 1.27 ms against 1.26.
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_F32
 #define CLOUDVOL_MARCH_MIN_BLOCKS_F32 6
 #endif
+#ifndef CLOUDVOL_MARCH_MIN_BLOCKS_F32_VIEWS
+#define CLOUDVOL_MARCH_MIN_BLOCKS_F32_VIEWS 5
+#endif
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_16
-#define CLOUDVOL_MARCH_MIN_BLOCKS_16 7
+#define CLOUDVOL_MARCH_MIN_BLOCKS_16 6
 #endif
 
 namespace cloudvol {
 
 // Records at the standard tile sizes and base tiles alone, 8 view steps per warp
-// iteration: 8 CTAs (64 registers, no spills; 1920x1080 x 8 steps, FP32: 83.4 us,
-// 83.3 with 7, 84.3 with 6, 86.5 with 9; 64 views, BF16: 10.50 ms, 10.73 with 7,
-// 10.96 with 6).  With 16 steps per iteration the per-warp scratch is 1.7x larger
+// iteration: 8 CTAs (64 registers; the 16-bit kernels of the standard sizes spill 4 to
+// 12 bytes in the multi-view and many-chunk marches, the FP32 ones of base tiles 4 to
+// 16, the others nothing; 1920x1080 x 8 steps, FP32: 83.4 us, 83.3 with 7, 84.3 with 6,
+// 86.5 with 9; 64 views, BF16: 10.50 ms, 10.73 with 7, 10.96 with 6).  With 16 steps per iteration the per-warp scratch is 1.7x larger
 // and 8 CTAs would leave the L1 28 KB: 7 CTAs for FP32 records and 6 for 16-bit
 // ones (64 views, BF16, by an earlier build: 18.7 ms against 19.5 ms with 8).
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX
@@ -57,11 +66,12 @@ namespace cloudvol {
 // value: compiled in, it gained nothing, and kept standard volumes with other
 // than six light steps (nine: 480 -> 431 us) from their own kernel.
 enum VolumeKind { kAnyVolume, kStandardVolume, kBaseVolume, kConstantVolume };
-template <typename T, int VOL, int CH>
+template <typename T, int VOL, int CH, bool VIEWS>
 struct MarchBlocks {
     static constexpr bool f32 = sizeof(T) == 4;
+    static constexpr int any_f32 = VIEWS ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_VIEWS : CLOUDVOL_MARCH_MIN_BLOCKS_F32;
     static constexpr int value =
-        VOL == kAnyVolume ? (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32 : CLOUDVOL_MARCH_MIN_BLOCKS_16)
+        VOL == kAnyVolume ? (f32 ? any_f32 : CLOUDVOL_MARCH_MIN_BLOCKS_16)
         : CH <= 8 ? (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX : CLOUDVOL_MARCH_MIN_BLOCKS_16_FX)
                   : (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX16 : CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16);
 };

@@ -10,7 +10,7 @@
 namespace cloudvol {
 
 template <typename T, int SHAPE, int VOL, int CH, int STEPS>
-__global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH>::value)
+__global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH, false>::value)
     march_kernel(const __grid_constant__ SceneParams p, const __grid_constant__ ViewParams v,
                  const T *__restrict__ base, const T *__restrict__ detail,
                  const T *__restrict__ weather, unsigned long long *__restrict__ counter) {
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH>::value)
 // is found by binary search over the views' first tile indices and staged in
 // shared memory.
 template <typename T, int SHAPE, int VOL, int CH>
-__global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH>::value)
+__global__ void __launch_bounds__(128, MarchBlocks<T, VOL, CH, true>::value)
     march_batch_kernel(const __grid_constant__ SceneParams p, const ViewParams *__restrict__ views,
                        int n_views, int total_tiles, unsigned int *__restrict__ work,
                        const T *__restrict__ base, const T *__restrict__ detail,
