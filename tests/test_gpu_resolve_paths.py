@@ -48,3 +48,14 @@ def test_tile_edges(api, oracle, w, h, fmt):
     sep = api.taa(_t(hist), _t(cur), m, history_fmt=fmt)
     fused = api.taa_reproject(vol, prm, prev, cam, _t(hist), _t(cur), history_fmt=fmt)
     assert torch.equal(sep, fused)
+
+
+# a first frame is the current frame in the history's format, whatever the motion
+@pytest.mark.parametrize("w,h", [(1, 1), (255, 1), (16, 16), (257, 1), (97, 61)])
+@pytest.mark.parametrize("fmt", ["fp32", "fp16"])
+def test_first_frame_is_the_current_frame(api, w, h, fmt):
+    import torch
+    rng = np.random.default_rng(w + h)
+    cur, mot = _t(I.synthetic_frame(rng, h, w)), _t(I.synthetic_motion(rng, h, w))
+    got = api.taa(None, cur, mot, history_fmt=fmt)
+    assert torch.equal(got, cur if fmt == "fp32" else cur.half())
