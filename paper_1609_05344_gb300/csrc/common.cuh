@@ -56,6 +56,8 @@ __device__ __forceinline__ bool in_range(unsigned *word, bool ok, unsigned site)
 }
 // Host: the current device's status word in checked builds, else nullptr.
 unsigned *check_word();
+// SMs of the current device (a GB300's 152 if the query fails).
+int sm_count();
 
 // ---------------------------------------------------------------------------
 // Counter-based hash: single-state PCG hash (Jarzynski & Olano, JCGT 2020):

@@ -162,8 +162,9 @@ __device__ __forceinline__ void motion_column(const MotionParams &p, int x, int 
 // Motions of kMotionRows vertically adjacent pixels of one column per thread:
 // the column terms are computed once and the rows' dependent chains (a
 // reciprocal square root and two reciprocals in series each) overlap; stores
-// stay coalesced along x.
-constexpr int kMotionRows = 4;
+// stay coalesced along x.  Four rows (1920x1080 5.8 us), or two where tiles of four
+// would leave SMs without a CTA (128x128: 1.6 us, with four 1.85).
+template <int kMotionRows>
 __global__ void __launch_bounds__(256) motion_kernel(const __grid_constant__ MotionParams p,
                                                      float2 *__restrict__ motion) {
     const int x = blockIdx.x * 32 + threadIdx.x;
@@ -499,14 +500,15 @@ __global__ void __launch_bounds__(256) first_frame_kernel(const float4 *__restri
 // kernel included, 32.8 us against 40.6 us for one pixel a thread with its
 // neighbours read through L1.  Two pixels and 4 / 5 CTAs 34.7 / 34.6
 // us with the motion, four pixels and 3 CTAs 38.0, one pixel and 6 CTAs 38.1
-// (before the prefetch).
-constexpr int kTaaPix = 2, kTaaBlocks = 4;
-template <typename H>
+// (before the prefetch).  One pixel a thread (kPix) where tiles of two would leave
+// SMs without a CTA: 128x128 FP16 2.1 us, with two 2.65.
+constexpr int kTaaBlocks = 4;
+template <typename H, int kPix>
 __global__ void __launch_bounds__(256, kTaaBlocks)
     taa_kernel(const H *__restrict__ hist, const float4 *__restrict__ cur,
                const float2 *__restrict__ mot, H *__restrict__ out, int W, int Hh, float blend,
                unsigned *check) {
-    constexpr int kPix = kTaaPix, kTH = 8 * kPix;
+    constexpr int kTH = 8 * kPix;
     __shared__ __align__(128) ResolveTile<kPix> tile;
     const int x0 = blockIdx.x * kTW, y0 = blockIdx.y * kTH;
     const int x = x0 + threadIdx.x, y = y0 + kPix * threadIdx.y;
@@ -659,9 +661,22 @@ int launch_motion(const cloud_volume *vol, const cloud_params *prm, const cloud_
     if (!aligned(motion, 8)) return set_error(CLOUD_ERR_INVALID_ARG, "cloud_motion: motion not 8-byte aligned");
     MotionParams p;
     if (int rc = build_motion_params(vol, prm, prev, cur, width, height, &p)) return rc;
-    const dim3 grid((width + 31) / 32, (height + 8 * kMotionRows - 1) / (8 * kMotionRows)), block(32, 8);
-    motion_kernel<<<grid, block, 0, s>>>(p, (float2 *)motion);
+    const int columns = (width + 31) / 32, rows = columns * ((height + 31) / 32) < sm_count() ? 2 : 4;
+    const dim3 grid(columns, (height + 8 * rows - 1) / (8 * rows)), block(32, 8);
+    if (rows == 2)
+        motion_kernel<2><<<grid, block, 0, s>>>(p, (float2 *)motion);
+    else
+        motion_kernel<4><<<grid, block, 0, s>>>(p, (float2 *)motion);
     return check_launch("motion_kernel");
+}
+
+template <typename H>
+static void launch_taa_kernel(const void *history, const float *current, const float *motion,
+                              void *history_out, int width, int height, int pix, float blend, cudaStream_t s) {
+    const dim3 grid((width + kTW - 1) / kTW, (height + 8 * pix - 1) / (8 * pix)), block(32, 8);
+    const auto kernel = pix == 1 ? taa_kernel<H, 1> : taa_kernel<H, 2>;
+    kernel<<<grid, block, 0, s>>>((const H *)history, (const float4 *)current, (const float2 *)motion,
+                                  (H *)history_out, width, height, blend, check_word());
 }
 
 int launch_taa(const void *history, const float *current, const float *motion, void *history_out,
@@ -691,16 +706,11 @@ int launch_taa(const void *history, const float *current, const float *motion, v
             first_frame_kernel<uint2><<<blocks, 256, 0, s>>>((const float4 *)current, (uint2 *)history_out, n);
         return check_launch("first_frame_kernel");
     }
-    const int rows = 8 * kTaaPix;
-    const dim3 grid((width + kTW - 1) / kTW, (height + rows - 1) / rows), block(32, 8);
+    const int columns = (width + kTW - 1) / kTW, pix = columns * ((height + 15) / 16) < sm_count() ? 1 : 2;
     if (fmt == CLOUD_HISTORY_FP32)
-        taa_kernel<float4><<<grid, block, 0, s>>>((const float4 *)history, (const float4 *)current,
-                                                  (const float2 *)motion, (float4 *)history_out,
-                                                  width, height, blend, check_word());
+        launch_taa_kernel<float4>(history, current, motion, history_out, width, height, pix, blend, s);
     else
-        taa_kernel<uint2><<<grid, block, 0, s>>>((const uint2 *)history, (const float4 *)current,
-                                                 (const float2 *)motion, (uint2 *)history_out,
-                                                 width, height, blend, check_word());
+        launch_taa_kernel<uint2>(history, current, motion, history_out, width, height, pix, blend, s);
     return check_launch("taa_kernel");
 }
 

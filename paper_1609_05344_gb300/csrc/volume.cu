@@ -52,6 +52,15 @@ unsigned *check_word() {
 #endif
 }
 
+int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+        return sms;
+    cudaGetLastError();
+    return 152;
+}
+
 __device__ __forceinline__ double unit_value(uint32_t h) {
     return (double)(h >> 8) * (1.0 / 16777216.0);
 }

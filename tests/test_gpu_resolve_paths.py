@@ -59,3 +59,24 @@ def test_first_frame_is_the_current_frame(api, w, h, fmt):
     cur, mot = _t(I.synthetic_frame(rng, h, w)), _t(I.synthetic_motion(rng, h, w))
     got = api.taa(None, cur, mot, history_fmt=fmt)
     assert torch.equal(got, cur if fmt == "fp32" else cur.half())
+
+
+# on both sides of the rules that give small images fewer pixels a thread: 152 tiles of
+# 32x32 pixels (motion) and of 32x16 (TAA), and the rows that a thread has beyond the image
+@pytest.mark.parametrize("w,h", [(31, 1), (33, 17), (608, 255), (609, 225), (304, 256), (577, 129), (640, 305)])
+@pytest.mark.parametrize("fmt", ["fp32", "fp16"])
+def test_small_images_resolve_as_large_ones(api, oracle, w, h, fmt):
+    import torch
+    rng = np.random.default_rng(w * h)
+    hist, cur = I.synthetic_frame(rng, h, w), I.synthetic_frame(rng, h, w)
+    hist = hist.astype(np.float16) if fmt == "fp16" else hist
+    desc, prm = I.volume_desc("tiny", seed=1), I.params()
+    prev, cam = I.orbit_camera(7, 3), I.orbit_camera(8, 3)
+    vol = api.Volume(desc)
+    mot = api.motion(vol, prm, prev, cam, w, h)
+    assert np.abs(mot.cpu().numpy() - oracle.motion(desc, prm, prev, cam, w, h)).max() <= 1e-4
+    got = api.taa(_t(hist), _t(cur), mot, history_fmt=fmt)
+    ref = oracle.taa(hist.astype(np.float64), cur, mot.cpu().numpy())
+    assert np.abs(got.cpu().numpy().astype(np.float64) - ref).max() <= (1e-6 if fmt == "fp32" else 2e-3)
+    fused = api.taa_reproject(vol, prm, prev, cam, _t(hist), _t(cur), history_fmt=fmt)
+    assert torch.equal(got, fused)
