@@ -129,7 +129,9 @@ struct SceneParams {
     // (mod 2^32), kfix = 2^32 / tile period.
     float2 kfix_h[kLatticeAxes], kfix_l[kLatticeAxes];   // each value twice (packed operands)
     uint32_t half_unit[kLatticeAxes];                    // half a texel: 2^(31 - log2 N)
-    uint32_t loff[CLOUD_MAX_LIGHT_STEPS][kLatticeAxes];  // light-sample offsets
+    // light-sample offsets; in standard volumes those of the detail axes are what is
+    // left of them once the base offset is shifted (see light_coords)
+    uint32_t loff[CLOUD_MAX_LIGHT_STEPS][kLatticeAxes];
     int32_t lh[CLOUD_MAX_LIGHT_STEPS];                   // light-sample height offsets
     int32_t h_top;                                       // layer thickness in 2^-16 m
     float h_lo_scale, h_hi_scale;  // 10/thickness, 2.5/thickness, per 2^-16 m
@@ -401,15 +403,17 @@ __device__ __forceinline__ Density density(const SceneParams &p, const T *__rest
     return {__fmul_rn(g, w), r};
 }
 
-// Coordinates of light sample j of a point (standard volumes: the detail
-// coordinates follow from the base ones).
+// Coordinates of light sample j of a point.  In standard volumes the detail
+// coordinates follow from the base ones by a multiply-add that also adds the
+// offset's rest in detail units, so that the offset is as exact as if it were added
+// to the point's own detail coordinates, which then need not be kept.
 template <int VOL>
 __device__ __forceinline__ void light_coords(const SceneParams &p, const uint32_t cs[kLatticeAxes], int j,
                                              uint32_t cj[kLatticeAxes]) {
 #pragma unroll
     for (int a = 0; a < kLatticeAxes; ++a)
-        cj[a] = VOL == kStandardVolume && a >= kDX && a <= kDZ ? mad32(cj[a - kDX], p.detail_mul, p.detail_add)
-                                           : mad32(cs[a], p.one, p.loff[j][a]);
+        cj[a] = VOL == kStandardVolume && a >= kDX && a <= kDZ ? mad32(cj[a - kDX], p.detail_mul, p.loff[j][a])
+                                                               : mad32(cs[a], p.one, p.loff[j][a]);
 }
 
 // Staging of one lane's start coordinates and increments (lattice axes, then

@@ -109,6 +109,10 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
         p->detail_mul = 1u << p->detail_shift;
         p->detail_add = (p->half_unit[kBX] << p->detail_shift) - p->half_unit[kDX];
     }
+    if (volume_kind(*p, vol) == kStandardVolume)
+        for (int j = 0; j < light_steps; ++j)
+            for (int a = kDX; a <= kDZ; ++a)
+                p->loff[j][a] += p->detail_add - p->loff[j][a - kDX] * p->detail_mul;
     p->base_mul[0] = 1u << vol->log2_base;
     p->base_mul[1] = 1u << (2 * vol->log2_base);
     p->detail_rec_mul[0] = 1u << vol->log2_detail;

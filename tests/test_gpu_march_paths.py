@@ -113,3 +113,28 @@ def test_constant_density(api, oracle, rho0, tau_max, integration, light_steps, 
     view = dict(camera=cam, width=w, height=h, steps=steps, jitter_frame=4)
     batch = api.Batch(vol, prm, [view, view], light_steps, integration)
     assert all(np.array_equal(o.cpu().numpy(), got.cpu().numpy()) for o in batch.render())
+
+
+# Light samples of a detail tile far finer than the base tile (2^k of its periods to one of the
+# base's) keep the detail tile's own precision.  Vertical one-pixel views at positions that fixed
+# point holds exactly, so that only the light offsets are rounded; opaque pixels (alpha >= 0.99),
+# whose colour is the sunlight of one step.  Relative tolerance: FP32 interpolation errs by at
+# most 1e-6 a density (three roundings of 2^-25 and weights of 2^-23 a tile, over 1 - c), the
+# optical depth of six samples of 0.04 x 37 by 9e-6, the exponential and the products by 1e-6.
+# A light offset rounded to a base unit is 1/4096 of a detail texel off at 2^16, up to 2e-4 here.
+@pytest.mark.parametrize("ratio", [8, 65536])
+def test_light_offsets_of_a_fine_detail_tile(api, oracle, ratio):
+    desc = I.volume_desc("full", seed=9, base_period=65536.0, detail_period=65536.0 / ratio,
+                         detail_weight=0.6, coverage=0.25)
+    prm = I.params(ambient=(0.0, 0.0, 0.0), light_step=37.0)
+    rng = np.random.default_rng(12)
+    views = [dict(camera=dict(pos=(x / 64.0, y / 64.0, 500.0), forward=(0.0, 0.0, 1.0),
+                              right=(1.0, 0.0, 0.0), up=(0.0, 1.0, 0.0), tan_half_fovy=0.5),
+                  width=1, height=1, steps=1, jitter_frame=-1)
+             for x, y in rng.integers(-2 ** 21, 2 ** 21, (256, 2))]
+    ovol = oracle.Volume(desc)
+    got = np.array([o.cpu().numpy()[0, 0] for o in api.Batch(api.Volume(desc), prm, views).render()])
+    ref = np.array([oracle.render(ovol, v["camera"], prm, 1, 1, 1, 6)[0][0, 0] for v in views])
+    opaque = ref[:, 3] >= 0.99
+    assert opaque.sum() >= 32
+    assert np.abs(got[opaque, :3] / ref[opaque, :3] - 1.0).max() <= 1e-5
