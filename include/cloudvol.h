@@ -250,16 +250,19 @@ int cloud_render_count(const cloud_volume *vol, const cloud_camera *cam, const c
  * 16x8, 1: 32x4 of 8x4-pixel warps, 2: 32x4 of 16x2-pixel warps, 3: 8x16) and
  * k selecting the view steps a warp evaluates per iteration of its march
  * (0: 8, 1: 16).  Every configuration gives bitwise the same pixels.  Until a
- * configuration is tuned or set, launches use 3 (8x16, 8 steps).  cloud_render
- * spreads images too small to fill the GPU (up to 77824 pixels) over more warps
- * than any configuration does, with the same pixels. */
+ * configuration is tuned or set, launches use 3 (8x16, 8 steps), and cloud_render
+ * spreads images too small to fill the GPU (up to 512 pixels an SM: 77824 with 152)
+ * over more warps than any configuration does, with the same pixels. */
 #define CLOUD_TUNE_CONFIGS 8
 
 /* Times every launch configuration of the raymarch on this workload (repeats
  * launches each, writing out_rgba), remembers the fastest for the volume's
  * storage precision and light-step count (later cloud_render, new batches and
  * new servers use it), and returns it in *best (and the per-configuration mean
- * times in times_ms[CLOUD_TUNE_CONFIGS] if not NULL).  Waits for the stream. */
+ * times in times_ms[CLOUD_TUNE_CONFIGS] if not NULL).  On an image too small to
+ * fill the GPU it also times the spread launch, and small images use that one
+ * unless *best was faster; a larger image leaves small ones to the spread launch.
+ * Waits for the stream. */
 int cloud_autotune_render(const cloud_volume *vol, const cloud_camera *cam, const cloud_params *prm,
                           int width, int height, int steps, int light_steps, int jitter_frame,
                           int integration, float *out_rgba, int repeats, float *times_ms,
@@ -268,6 +271,8 @@ int cloud_autotune_render(const cloud_volume *vol, const cloud_camera *cam, cons
 /* Reads / sets the launch configuration that cloud_render, new batches and
  * new servers use for volumes of `precision` rendered with `light_steps`
  * light steps (e.g. to restore a configuration an earlier autotune found).
+ * A configuration that is set applies to images of every size; setting the
+ * default (3) restores the initial state, small images spread over more warps.
  * config outside [0, CLOUD_TUNE_CONFIGS) or a bad precision is
  * CLOUD_ERR_INVALID_ARG.  Process-wide; host only.
  * Scheduling only; no counterpart in the paper (the pixel results do not

@@ -190,12 +190,16 @@ int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_cam
 }
 
 // ---------------------------------------------------------------------------
-// Launch-configuration selection: the autotuner records the fastest (tile
-// shape, view steps per warp iteration) per (storage precision, six light steps
-// or another number); launches use it when present.
+// Launch-configuration selection per (storage precision, six light steps or another
+// number): what the autotuner found fastest or the caller set, -1 for the default.  A
+// single view too small to fill the GPU has a choice of its own: -1 leaves it to
+// small_shape below, which the eight configurations hardly ever beat there.
 namespace {
-std::mutex g_tune_mu;
-int g_best_config[4][2] = {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}};
+struct Choice {
+    int config = -1, small = -1;
+};
+std::mutex g_choice_mu;
+Choice g_choice[4][2];
 }  // namespace
 
 // Untuned default: shape 3 (8x16-pixel CTA of 4x8-pixel warps), 8 view steps
@@ -203,14 +207,19 @@ int g_best_config[4][2] = {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}};
 // precision measured.
 constexpr int kDefaultConfig = 3;
 
-int tuned_config(int precision, int light_steps) {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    const int c = g_best_config[precision & 3][light_steps == 6 ? 1 : 0];
-    return c < 0 ? kDefaultConfig : c;
+static Choice choice(int precision, int light_steps) {
+    std::lock_guard<std::mutex> lk(g_choice_mu);
+    return g_choice[precision & 3][light_steps == 6 ? 1 : 0];
 }
-void set_tuned_config(int precision, int light_steps, int config) {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_best_config[precision & 3][light_steps == 6 ? 1 : 0] = config;
+static void set_choice(int precision, int light_steps, int config, int small) {
+    std::lock_guard<std::mutex> lk(g_choice_mu);
+    Choice &c = g_choice[precision & 3][light_steps == 6 ? 1 : 0];
+    c.config = config;
+    c.small = small;
+}
+int tuned_config(int precision, int light_steps) {
+    const int c = choice(precision, light_steps).config;
+    return c < 0 ? kDefaultConfig : c;
 }
 
 // Tile shape of a single view too small to fill the GPU, or -1.  Below one wave
@@ -254,7 +263,10 @@ int launch_render(const cloud_volume *vol, const cloud_camera *cam, const cloud_
         return set_error(CLOUD_ERR_INVALID_ARG, "cloud_render: counter not 8-byte aligned");
     SceneParams p;
     ViewParams v;
-    const int config = tuned_config(vol->desc.precision, light_steps), small = small_shape(width, height);
+    const Choice chosen = choice(vol->desc.precision, light_steps);
+    const int rule = small_shape(width, height);  // a configuration chosen for small views overrides it
+    const int small = chosen.small < 0 ? rule : -1, pick = rule < 0 ? chosen.config : chosen.small;
+    const int config = pick < 0 ? kDefaultConfig : pick;
     if (int rc = build_scene(vol, prm, light_steps, integration, &p)) return rc;
     if (int rc = build_view(vol, prm, cam, width, height, steps, jitter_frame, out,
                             small >= 0 ? small : config_shape(config), &v))
@@ -304,31 +316,44 @@ extern "C" int cloud_autotune_render(const cloud_volume *vol, const cloud_camera
         cudaEventDestroy(e0);
         return rc;
     }
-    int best_config = 0, rc = CLOUD_OK;
-    float best_ms = INFINITY;
-    for (int config = 0; config < kConfigs && !rc; ++config) {
+    int best_config = 0;
+    float best_ms = INFINITY, rule_ms = INFINITY;
+    // mean time of a launch with configuration `config`, or with small shape `rule`
+    const auto time_launches = [&](int config, int rule, float *ms) -> int {
         ViewParams v;
-        rc = build_view(vol, prm, cam, width, height, steps, jitter_frame, out_rgba,
-                        config_shape(config), &v);
-        if (rc) break;
-        rc = launch_march(p, v, vol, nullptr, config, s);  // warm-up
+        if (int rc = build_view(vol, prm, cam, width, height, steps, jitter_frame, out_rgba,
+                                rule >= 0 ? rule : config_shape(config), &v))
+            return rc;
+        const auto launch = [&]() -> int {
+            if (rule < 0) return launch_march(p, v, vol, nullptr, config, s);
+            launch_march_small(p, v, vol, nullptr, rule, s);
+            return check_launch("march_kernel");
+        };
+        int rc = launch();  // warm-up
         if (!rc) rc = check_cuda(cudaEventRecord(e0, s), "cudaEventRecord");
-        for (int r = 0; r < repeats && !rc; ++r) rc = launch_march(p, v, vol, nullptr, config, s);
+        for (int r = 0; r < repeats && !rc; ++r) rc = launch();
         if (!rc) rc = check_cuda(cudaEventRecord(e1, s), "cudaEventRecord");
         if (!rc) rc = check_cuda(cudaEventSynchronize(e1), "cudaEventSynchronize");
+        if (!rc) rc = check_cuda(cudaEventElapsedTime(ms, e0, e1), "cudaEventElapsedTime");
+        *ms /= repeats;
+        return rc;
+    };
+    int rc = CLOUD_OK;
+    for (int config = 0; config < kConfigs && !rc; ++config) {
         float ms = 0.0f;
-        if (!rc) rc = check_cuda(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
-        ms /= repeats;
-        if (times_ms) times_ms[config] = ms;
+        rc = time_launches(config, -1, &ms);
+        if (!rc && times_ms) times_ms[config] = ms;
         if (!rc && ms < best_ms) {
             best_ms = ms;
             best_config = config;
         }
     }
+    const int rule = small_shape(width, height);
+    if (!rc && rule >= 0) rc = time_launches(0, rule, &rule_ms);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
-    set_tuned_config(vol->desc.precision, light_steps, best_config);
+    set_choice(vol->desc.precision, light_steps, best_config, rule >= 0 && best_ms < rule_ms ? best_config : -1);
     if (best) *best = best_config;
     return CLOUD_OK;
 }
@@ -346,7 +371,7 @@ extern "C" int cloud_set_launch_config(int precision, int light_steps, int confi
     if (precision < CLOUD_PRECISION_FP32 || precision > CLOUD_PRECISION_UNORM16 || config < 0 ||
         config >= kConfigs)
         return set_error(CLOUD_ERR_INVALID_ARG, "cloud_set_launch_config: bad arguments");
-    set_tuned_config(precision, light_steps, config);
+    set_choice(precision, light_steps, config, config == kDefaultConfig ? -1 : config);
     return CLOUD_OK;
 }
 

@@ -4,6 +4,8 @@ the layer, step counts that do not fill a chunk, and rays in clear air.
 
 Tolerances (max-abs RGBA) are those of every other render: 1e-4 for FP32
 volumes, 3e-3 for FP16 volumes."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -138,3 +140,85 @@ def test_light_offsets_of_a_fine_detail_tile(api, oracle, ratio):
     opaque = ref[:, 3] >= 0.99
     assert opaque.sum() >= 32
     assert np.abs(got[opaque, :3] / ref[opaque, :3] - 1.0).max() <= 1e-5
+
+
+class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("shared", ctypes.c_uint), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def _grid(launch):
+    """Grid (x, y) of the one kernel that launch(stream) issues, captured and not run."""
+    import torch
+    cu, s = ctypes.CDLL("libcuda.so.1"), torch.cuda.Stream()
+    handle, graph, node, n = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_size_t(1)
+    assert cu.cuStreamBeginCapture_v2(handle, 2) == 0
+    try:
+        launch(s)
+    finally:
+        assert cu.cuStreamEndCapture(handle, ctypes.byref(graph)) == 0
+    got = _KernelNode()
+    assert cu.cuGraphGetNodes(graph, ctypes.byref(node), ctypes.byref(n)) == 0 and n.value == 1
+    assert cu.cuGraphKernelNodeGetParams_v2(node, ctypes.byref(got)) == 0
+    cu.cuGraphDestroy(graph)
+    return tuple(got.grid[:2])
+
+
+TILES = [(16, 8), (32, 4), (32, 4), (8, 16)]  # of the four shapes
+
+
+def _tiles(config, w, h):
+    tw, th = TILES[config % 4]
+    return (w + tw - 1) // tw, (h + th - 1) // th
+
+
+# a configuration that is set reaches images of every size, the default gives small ones back
+# to the rule (8x4 tiles at 203x77), and tuning on one size leaves the other in order
+def test_launch_config_reaches_every_size(api):
+    import torch
+    vol, cam, prm = api.Volume(I.volume_desc("full", seed=3, precision="fp16")), I.orbit_camera(2, 3), I.params()
+    sizes = [(203, 77), (411, 203)]
+    outs = [torch.empty((h, w, 4), device="cuda") for w, h in sizes]
+
+    def grid(k):
+        return _grid(lambda s: api.render(vol, cam, prm, *sizes[k], 8, 6, jitter_frame=1, out=outs[k], stream=s))
+
+    spread = (26, 20)
+    api.set_launch_config("fp16", 6, 3)
+    try:
+        assert grid(0) == spread and grid(1) == _tiles(3, *sizes[1])
+        for config in (0, 1, 2, 4, 5, 6, 7):
+            api.set_launch_config("fp16", 6, config)
+            assert api.launch_config("fp16", 6) == config
+            assert [grid(0), grid(1)] == [_tiles(config, *s) for s in sizes]
+        best, _ = api.autotune_render(vol, cam, prm, *sizes[1], 8, 6, jitter_frame=1, repeats=2)
+        assert api.launch_config("fp16", 6) == best
+        assert grid(0) == spread and grid(1) == _tiles(best, *sizes[1])
+        best, _ = api.autotune_render(vol, cam, prm, *sizes[0], 8, 6, jitter_frame=1, repeats=2)
+        assert api.launch_config("fp16", 6) == best and grid(1) == _tiles(best, *sizes[1])
+        assert grid(0) in (spread, _tiles(best, *sizes[0]))
+    finally:
+        api.set_launch_config("fp16", 6, 3)
+    assert grid(0) == spread
+
+
+# every configuration on an image above the rule for small ones, in marches of one chunk, of
+# several and of a part, for the kernels of each kind of volume
+@pytest.mark.parametrize("kind,precision,over", [("full", "fp32", {}), ("full", "bf16", {}), ("tiny", "fp32", {}),
+                                                 ("tiny", "unorm16", {}), ("full", "fp16", dict(base_n=64)),
+                                                 ("constant", "fp32", {})])
+@pytest.mark.parametrize("steps", [8, 40])
+def test_every_launch_config_on_a_large_image(api, kind, precision, over, steps):
+    import torch
+    vol = api.Volume(I.volume_desc(kind, seed=3, precision=precision, **over))
+    cam, outs = I.orbit_camera(2, 3), []
+    try:
+        for config in range(8):
+            api.set_launch_config(precision, 6, config)
+            outs.append(api.render(vol, cam, I.params(), 411, 203, steps, 6, jitter_frame=1))
+    finally:
+        api.set_launch_config(precision, 6, 3)
+    assert outs[0][..., 3].max() > 0.1
+    for config in range(1, 8):
+        assert torch.equal(outs[0], outs[config]), config
