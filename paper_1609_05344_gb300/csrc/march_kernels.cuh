@@ -82,8 +82,9 @@ void launch_shape(const SceneParams &p, const ViewParams &v, const cloud_volume 
             march_kernel<T, SHAPE, kBaseVolume, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
             break;
         case kConstantVolume:
-            march_kernel<float, SHAPE, kConstantVolume, CH, kAnySteps>
-                <<<grid, 128, 0, s>>>(p, v, nullptr, nullptr, nullptr, counter);
+            if constexpr (SHAPE < kShapes)  // never spread over more warps (small_shape)
+                march_kernel<float, SHAPE, kConstantVolume, CH, kAnySteps>
+                    <<<grid, 128, 0, s>>>(p, v, nullptr, nullptr, nullptr, counter);
             break;
         default: march_kernel<T, SHAPE, kAnyVolume, CH, kAnySteps><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);
     }

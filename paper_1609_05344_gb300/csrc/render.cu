@@ -222,17 +222,24 @@ int tuned_config(int precision, int light_steps) {
     return c < 0 ? kDefaultConfig : c;
 }
 
-// Tile shape of a single view too small to fill the GPU, or -1.  Below one wave
-// of warps (32 on each of the 152 SMs) a launch is a chain of latencies, shorter
-// the fewer rays share a warp's lookups: 8 or 16 rays a warp while that still
-// fits one wave, 4 up to half a wave (their setup wastes more lanes than it
-// gains beyond).  GPU time, 32 / 16 / 8 / 4 rays a warp, 64 steps, FP32, full
+// Tile shape of a single view too small to fill the GPU, or -1.  Below one wave of
+// warps (32 an SM, what the kernels of standard and base-only volumes keep resident) a
+// launch is a chain of latencies, shorter the fewer rays share a warp's lookups: 8 or 16
+// rays a warp while that still fits one wave, 4 up to half a wave (their setup wastes
+// more lanes than it gains beyond).  GPU time, 32 / 16 / 8 / 4 rays a warp, 64 steps, FP32, full
 // tiles: 64x64 62.0 / 44.7 / 32.4 / 28.9 us, 128x128 69.5 / 46.3 / 35.0 / 35.6,
 // 200x160 71.2 / 50.3 / 41.0 / 53.2, 320x240 78.4 / 60.3 / 69.6 / 92.3; 8 steps:
 // 9.9 / 7.9 / 5.9 / 5.9, 11.3 / 8.2 / 6.8 / 8.5, 11.7 / 9.1 / 8.9 / 13.0, 13.2 /
-// 11.9 / 15.6 / 23.7; 640x360 x 8 steps 23.1 / 24.9 / 35.8.
-static int small_shape(int width, int height) {
-    const int64_t wave = 152 * 32, pixels = (int64_t)width * height;
+// 11.9 / 15.6 / 23.7; 640x360 x 8 steps 23.1 / 24.9 / 35.8.  Volumes of any tile sizes
+// keep 24 warps an SM, but the same limits serve them: 304x256 (16 rays) against
+// 307x257 (32) FP32 11.7 / 14.0 us at 8 steps and 60 / 81 at 64, FP16 12.1 / 14.5 and
+// 61 / 84, a detail tile of another period 14.8 / 16.6 and 75 / 96; base-only FP16
+// 11.5 / 13.0 and 56 / 72.  The one exception measured: UNORM16 standard volumes at
+// 8 steps, 13.1 / 12.9 (64 steps 73 / 80).  Constant density has no lookups to share:
+// 304x256 x 8 steps 3.7 us with 16 rays a warp, 2.8 with 32; 64x64 2.5 / 2.2.
+static int small_shape(const cloud_volume *vol, int width, int height) {
+    if (vol->desc.density_mode != CLOUD_DENSITY_NOISE) return -1;
+    const int64_t wave = 32 * sm_count(), pixels = (int64_t)width * height;
     return pixels <= 2 * wave ? 6 : pixels <= 8 * wave ? 5 : pixels <= 16 * wave ? 4 : -1;
 }
 
@@ -264,7 +271,7 @@ int launch_render(const cloud_volume *vol, const cloud_camera *cam, const cloud_
     SceneParams p;
     ViewParams v;
     const Choice chosen = choice(vol->desc.precision, light_steps);
-    const int rule = small_shape(width, height);  // a configuration chosen for small views overrides it
+    const int rule = small_shape(vol, width, height);  // a configuration chosen for small views overrides it
     const int small = chosen.small < 0 ? rule : -1, pick = rule < 0 ? chosen.config : chosen.small;
     const int config = pick < 0 ? kDefaultConfig : pick;
     if (int rc = build_scene(vol, prm, light_steps, integration, &p)) return rc;
@@ -348,7 +355,7 @@ extern "C" int cloud_autotune_render(const cloud_volume *vol, const cloud_camera
             best_config = config;
         }
     }
-    const int rule = small_shape(width, height);
+    const int rule = small_shape(vol, width, height);
     if (!rc && rule >= 0) rc = time_launches(0, rule, &rule_ms);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
