@@ -30,7 +30,7 @@ int launch_batch(const cloud_volume *vol, const SceneParams &scene, const ViewPa
                  int n_views, int total_tiles, int config, unsigned int *d_work,
                  unsigned long long *counter, cudaStream_t s) {
     if (total_tiles == 0) return CLOUD_OK;
-    const void *fn = batch_kernel(vol->desc.precision, volume_kind(scene, vol), config);
+    const void *fn = batch_kernel(vol->desc.precision, volume_kind(vol), config);
     int dev = 0, sms = 0, per_sm = 0;
     if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
     if (int rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev),

@@ -100,7 +100,7 @@ struct cloud_volume {
     // occupancy grid: one bit per cell of 2^kOccShift base records per axis (x fastest),
     // clear where the density is provably 0 throughout (see build_occupancy)
     uint32_t *occ;   // device or nullptr (constant density)
-    uint32_t *occ_blocks;  // the same bits in blocks of 16^3 cells, or nullptr (not 256^3 cells)
+    uint32_t *occ_blocks;  // the same bits in blocks of 16^3 cells (standard volumes), or nullptr
     int log2_occ;    // macro-cells per axis = 2^log2_occ = base_n / 2^kOccShift
     int device;
 };
@@ -111,6 +111,32 @@ inline int ilog2(int n) {
     int l = 0;
     while ((1 << l) < n) ++l;
     return l;
+}
+
+// The standard tile sizes (128^3 base, 32^3 detail, 512^2 weather records) as
+// compile-time constants: the record-index and weight shifts of every
+// lookup are immediates instead of per-launch values.
+constexpr int kStdLog2Base = 7, kStdLog2Detail = 5, kStdLog2Weather = 9;
+
+// What a march is compiled for: any volume of noise tiles; the standard tile sizes
+// (below); a base tile of any size alone, with neither detail nor weather, which
+// needs a third of the records and registers for 8 CTAs (64^3 base, 1280x720 x 64
+// steps 520.7 us as any volume, 307.5 as this); constant density (FP32 kernels
+// only: it has no records).  The number of light steps is a launch
+// value: compiled in, it gained nothing, and kept standard volumes with other
+// than six light steps (nine: 480 -> 431 us) from their own kernel.
+enum VolumeKind { kAnyVolume, kStandardVolume, kBaseVolume, kConstantVolume };
+// The kind of march of a volume: standard needs the standard tile sizes, all three
+// tiles and a base tile period of 2^k detail periods (the detail coordinates then
+// follow from the base ones); base neither a detail nor a weather tile; constant no
+// tile at all.
+int volume_kind(const cloud_volume *vol);
+// k where the base tile period is 2^k detail periods (0 <= k <= 16), else -1.
+inline int detail_shift(const cloud_volume_desc &d) {
+    const double ratio = d.base_period_m / d.detail_period_m;
+    for (int k = 0; k <= 16; ++k)
+        if (ratio == (double)(1 << k)) return k;
+    return -1;
 }
 
 inline size_t precision_bytes(int p) { return p == CLOUD_PRECISION_FP32 ? 4 : 2; }

@@ -58,14 +58,6 @@ namespace cloudvol {
 #ifndef CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16
 #define CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16 6
 #endif
-// What a march is compiled for: any volume of noise tiles; the standard tile sizes
-// (below); a base tile of any size alone, with neither detail nor weather, which
-// needs a third of the records and registers for 8 CTAs (64^3 base, 1280x720 x 64
-// steps 520.7 us as any volume, 307.5 as this); constant density (FP32 kernels
-// only: it has no records).  The number of light steps is a launch
-// value: compiled in, it gained nothing, and kept standard volumes with other
-// than six light steps (nine: 480 -> 431 us) from their own kernel.
-enum VolumeKind { kAnyVolume, kStandardVolume, kBaseVolume, kConstantVolume };
 template <typename T, int VOL, int CH, bool VIEWS>
 struct MarchBlocks {
     static constexpr bool f32 = sizeof(T) == 4;
@@ -75,11 +67,6 @@ struct MarchBlocks {
         : CH <= 8 ? (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX : CLOUDVOL_MARCH_MIN_BLOCKS_16_FX)
                   : (f32 ? CLOUDVOL_MARCH_MIN_BLOCKS_F32_FX16 : CLOUDVOL_MARCH_MIN_BLOCKS_16_FX16);
 };
-
-// The standard tile sizes (128^3 base, 32^3 detail, 512^2 weather records) as
-// compile-time constants: the record-index and weight shifts of every
-// lookup are immediates instead of per-launch values.
-constexpr int kStdLog2Base = 7, kStdLog2Detail = 5, kStdLog2Weather = 9;
 
 // Light samples of a march evaluated per iteration of the light loop (the
 // density code is inlined that many times): one for FP32 records, whose three
@@ -897,10 +884,5 @@ void launch_march_small(const SceneParams &p, const ViewParams &v, const cloud_v
                         unsigned long long *counter, int shape, cudaStream_t s);
 template <int CH>
 const void *batch_kernel_ch(int precision, int kind, int shape);
-// The kind of march a launch takes: standard needs the standard tile sizes, all
-// three tiles and a base tile period of 2^k detail periods (the detail coordinates
-// then follow from the base ones); base neither a detail nor a weather tile;
-// constant no tile at all.
-int volume_kind(const SceneParams &p, const cloud_volume *vol);
 
 }  // namespace cloudvol

@@ -71,7 +71,7 @@ void launch_shape(const SceneParams &p, const ViewParams &v, const cloud_volume 
     tile_dims(SHAPE, &tw, &th);
     const dim3 grid(v.tiles_x, (v.height + th - 1) / th);
     const T *b = (const T *)vol->base, *d = (const T *)vol->detail, *w = (const T *)vol->weather;
-    switch (volume_kind(p, vol)) {
+    switch (volume_kind(vol)) {
         case kStandardVolume:
             if (v.steps <= CH)
                 march_kernel<T, SHAPE, kStandardVolume, CH, kOneChunk><<<grid, 128, 0, s>>>(p, v, b, d, w, counter);

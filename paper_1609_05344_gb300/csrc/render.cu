@@ -99,17 +99,12 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
     if (noise && vol->log2_detail) least_period = std::min(least_period, d.detail_period_m);
     if (noise && vol->log2_weather) least_period = std::min(least_period, d.weather_period_m);
     p->wide = noise && !(prm->t_max_m < 1000.0 * least_period);
-    p->detail_shift = -1;
-    if (vol->log2_detail) {
-        const double ratio = d.base_period_m / d.detail_period_m;
-        for (int k = 0; k <= 16; ++k)
-            if (ratio == std::ldexp(1.0, k)) p->detail_shift = k;
-    }
+    p->detail_shift = vol->log2_detail ? detail_shift(d) : -1;
     if (p->detail_shift >= 0) {
         p->detail_mul = 1u << p->detail_shift;
         p->detail_add = (p->half_unit[kBX] << p->detail_shift) - p->half_unit[kDX];
     }
-    if (volume_kind(*p, vol) == kStandardVolume)
+    if (volume_kind(vol) == kStandardVolume)
         for (int j = 0; j < light_steps; ++j)
             for (int a = kDX; a <= kDZ; ++a)
                 p->loff[j][a] += p->detail_add - p->loff[j][a - kDX] * p->detail_mul;
@@ -243,11 +238,11 @@ static int small_shape(const cloud_volume *vol, int width, int height) {
     return pixels <= 2 * wave ? 6 : pixels <= 8 * wave ? 5 : pixels <= 16 * wave ? 4 : -1;
 }
 
-int volume_kind(const SceneParams &p, const cloud_volume *vol) {
+int volume_kind(const cloud_volume *vol) {
     if (vol->desc.density_mode != CLOUD_DENSITY_NOISE) return kConstantVolume;
     if (!vol->detail && !vol->weather) return kBaseVolume;
-    return vol->detail && vol->weather && p.log2_base == kStdLog2Base && p.log2_detail == kStdLog2Detail &&
-                   p.log2_weather == kStdLog2Weather && p.detail_shift >= 0
+    return vol->detail && vol->weather && vol->log2_base == kStdLog2Base && vol->log2_detail == kStdLog2Detail &&
+                   vol->log2_weather == kStdLog2Weather && detail_shift(vol->desc) >= 0
                ? kStandardVolume
                : kAnyVolume;
 }

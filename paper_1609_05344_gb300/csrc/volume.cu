@@ -512,9 +512,13 @@ int build_occupancy(cloud_volume *v, cudaStream_t s) {
             (const T *)v->base, v->log2_base, (const T *)v->detail, v->log2_detail, (float)ratio, range[0],
             range[1], k0, (float)wd, v->occ);
     if (int rc = check_launch("occupancy_kernel")) return rc;
-    if (v->log2_occ != 8) return CLOUD_OK;
-    if (int rc = check_cuda(cudaMalloc(&v->occ_blocks, words * sizeof(uint32_t)), "cudaMalloc occupancy blocks"))
-        return rc;
+    // the copy is for the marches of standard volumes, which do without it as well
+    if (v->log2_occ != 8 || volume_kind(v) != kStandardVolume) return CLOUD_OK;
+    if (cudaMalloc(&v->occ_blocks, words * sizeof(uint32_t)) != cudaSuccess) {
+        cudaGetLastError();
+        v->occ_blocks = nullptr;
+        return CLOUD_OK;
+    }
     occupancy_blocks_kernel<<<(unsigned)(words / 256), 256, 0, s>>>(v->occ, v->occ_blocks);
     return check_launch("occupancy_blocks_kernel");
 }

@@ -222,3 +222,17 @@ def test_every_launch_config_on_a_large_image(api, kind, precision, over, steps)
     assert outs[0][..., 3].max() > 0.1
     for config in range(1, 8):
         assert torch.equal(outs[0], outs[config]), config
+
+
+# only standard volumes hold the blocked copy of the occupancy grid (2 MiB): a base tile of the
+# standard size alone is 32 MiB of 16-bit records and 2 MiB of grid
+def test_blocked_grid_only_where_it_is_read(api):
+    import torch
+    torch.cuda.synchronize()
+    first = api.Volume(I.volume_desc("tiny", seed=1, precision="fp16", base_n=128))  # loads the kernels
+    before = torch.cuda.mem_get_info()[0]
+    more = [api.Volume(I.volume_desc("tiny", seed=k, precision="fp16", base_n=128)) for k in range(16)]
+    used = (before - torch.cuda.mem_get_info()[0]) / len(more) / 2 ** 20
+    assert 33.5 <= used <= 35.0
+    for v in [first] + more:
+        v.close()
