@@ -112,10 +112,9 @@ enum Axis { kBX = 0, kBY, kBZ, kDX, kDY, kDZ, kWX, kWY, kLatticeAxes };
 
 // Constants shared by every view of a launch: volume, lighting, light march.
 struct SceneParams {
-    // Fixed-point lattice coordinates: coordinate = p * kfix - half_unit
+    // Fixed-point lattice coordinates: coordinate = p * kfix - half a texel
     // (mod 2^32), kfix = 2^32 / tile period.
     float2 kfix_h[kLatticeAxes], kfix_l[kLatticeAxes];   // each value twice (packed operands)
-    uint32_t half_unit[kLatticeAxes];                    // half a texel: 2^(31 - log2 N)
     // light-sample offsets; in standard volumes those of the detail axes are what is
     // left of them once the base offset is shifted (see light_coords)
     uint32_t loff[CLOUD_MAX_LIGHT_STEPS][kLatticeAxes];
@@ -137,7 +136,7 @@ struct SceneParams {
     unsigned *check;  // status word of the checked build, else nullptr
     int log2_base, log2_detail, log2_weather;
     int light_steps, integration;
-    int wide;  // t_max spans more than 1000 tile periods (df_to_u32)
+    int wide;  // t_max spans more than 1000 tile periods (df2_to_u32)
     // detail coordinates = base detail_mul + detail_add (mod 2^32) when the base
     // tile period is 2^detail_shift detail periods (-1: convert separately)
     int detail_shift;
@@ -155,7 +154,7 @@ struct ViewParams {
     // Camera rays, unnormalised: v(x, y) = v00 + x vx + y vy, as double-float
     // pairs; vx/vy are split so that x * hi is exact (see split_df10).
     float v00h[3], v00l[3], vxh[3], vxl[3], vyh[3], vyl[3];
-    // camera position in fixed-point lattice coordinates (half_unit taken off) and
+    // camera position in fixed-point lattice coordinates (half a texel taken off) and
     // its height above the layer bottom in 2^-16 m, each as the nearest integer and
     // the rest (in [-1/2, 1/2]): a sample's coordinate is rounded once, from the sum
     uint32_t org[kLatticeAxes], org_h;

@@ -58,7 +58,6 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
         split_df(kfix, &p->kfix_h[a].x, &p->kfix_l[a].x);
         p->kfix_h[a].y = p->kfix_h[a].x;
         p->kfix_l[a].y = p->kfix_l[a].x;
-        p->half_unit[a] = 1u << (31 - L[a]);
         for (int j = 0; j < light_steps; ++j) {
             const double off = (j + 0.5) * prm->light_step_m * s[comp] * kfix;
             p->loff[j][a] = (uint32_t)(unsigned long long)std::llrint(off);
@@ -102,7 +101,8 @@ int build_scene(const cloud_volume *vol, const cloud_params *prm, int light_step
     p->detail_shift = vol->log2_detail ? detail_shift(d) : -1;
     if (p->detail_shift >= 0) {
         p->detail_mul = 1u << p->detail_shift;
-        p->detail_add = (p->half_unit[kBX] << p->detail_shift) - p->half_unit[kDX];
+        // half a texel of each tile: 2^(31 - log2 N) units
+        p->detail_add = (1u << (31 - vol->log2_base) << p->detail_shift) - (1u << (31 - vol->log2_detail));
     }
     if (volume_kind(vol) == kStandardVolume)
         for (int j = 0; j < light_steps; ++j)

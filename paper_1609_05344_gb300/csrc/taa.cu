@@ -27,7 +27,7 @@ struct MotionParams {
     float G[3][3], dlt[3];
     float kx, ky, kx1, ky1;  // aT'/aT, T'/T, and the same minus 1
     float sx, sy;            // W / (2 aT'), H / (2 T')
-    int width, height, cam_in_layer;
+    int width, height;
     // double-float restatement of the world-space ray for near-tie layer-entry
     // decisions: v(x, y) = v00 + x vx + y vy (vx, vy split so that x * hi is
     // exact), slab_lo - o_z, slab_hi - o_z and the far clip
@@ -316,7 +316,7 @@ struct Footprints {
     bool use[kPix];    // the pixel has history on screen
     float4 hf[kPix];   // its filtered value
 
-    // mot(r, &m) gives the motion of pixel (x, y0 + r)
+    // mot(r) gives the motion of pixel (x, y0 + r)
     template <typename Motion>
     __device__ __forceinline__ void gather(const H *__restrict__ hist, int x, int y0, int W, int Hh,
                                            unsigned *check, const Motion &mot) {
@@ -639,7 +639,6 @@ int build_motion_params(const cloud_volume *vol, const cloud_params *prm, const 
     p->sy = (float)(height / (2.0 * Tp));
     p->width = width;
     p->height = height;
-    p->cam_in_layer = cur->pos[2] >= vol->desc.slab_lo_m && cur->pos[2] <= vol->desc.slab_hi_m;
     const double a0 = (1.0 / width - 1.0) * aT, ax = 2.0 * aT / width;
     const double b0 = (1.0 - 1.0 / height) * T, by = -2.0 * T / height;
     for (int k = 0; k < 3; ++k) {
