@@ -13,11 +13,18 @@ import torch
 from . import _native as N
 
 
+# The current device and its stream's handle without a Stream object (most of a short
+# call's own host time otherwise).  Not part of torch's public interface: a torch without
+# them goes through torch.cuda.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+
+
 def _stream(stream=None) -> int:
     if stream is not None:
         return stream.cuda_stream
-    if torch.cuda.is_initialized():  # the handle alone, without a Stream object
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(_device())
     return torch.cuda.current_stream().cuda_stream
 
 
@@ -30,7 +37,7 @@ def _require_cuda(t: torch.Tensor, name: str, dtype=None, shape=None):
     current device: anything else is refused here, before a launch."""
     if not isinstance(t, torch.Tensor) or not t.is_cuda or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous CUDA tensor")
-    if t.get_device() != torch._C._cuda_getDevice():
+    if t.get_device() != _device():
         raise ValueError(f"{name} is on {t.device}, the current device is "
                          f"cuda:{torch.cuda.current_device()}")
     if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
