@@ -9,6 +9,7 @@
 // interpolation; voxel k holds the noise at lattice coordinate k M_o / N.
 // The generation arithmetic runs in FP64 on the device so every stored texel
 // is the correctly rounded fBm value (minus the 1/2 centring offset).
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -53,12 +54,13 @@ unsigned *check_word() {
 }
 
 int sm_count() {
+    static std::atomic<int> known[64];  // asked once a device: the query costs a short call 3 % of its time
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
-        return sms;
-    cudaGetLastError();
-    return 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    if ((sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 152;
+    known[dev].store(sms, std::memory_order_relaxed);
+    return sms;
 }
 
 __device__ __forceinline__ double unit_value(uint32_t h) {
