@@ -1,7 +1,7 @@
 """GPU parity of the resolve kernels at the edges of their tiles: images one
 pixel short of, equal to and one past the tiles of 32x16 and 32x32 pixels, the
 separate motion and TAA passes against the FP64 oracle and the fused resolve
-bitwise against both, and the composite on both sides of its size rule.
+bitwise against both, and the composite at the edges of its 32x8 tiles.
 
 Tolerances: motion 1e-4 px, FP32 history 1e-6, FP16 history its storage rounding
 (2e-3 for values up to 2), composite 2e-6 (values up to 2)."""
@@ -80,3 +80,16 @@ def test_small_images_resolve_as_large_ones(api, oracle, w, h, fmt):
     assert np.abs(got.cpu().numpy().astype(np.float64) - ref).max() <= (1e-6 if fmt == "fp32" else 2e-3)
     fused = api.taa_reproject(vol, prm, prev, cam, _t(hist), _t(cur), history_fmt=fmt)
     assert torch.equal(got, fused)
+
+
+# one pixel, one short of, equal to and one past the 32x8 tiles; the cloud at the display's size,
+# odd fractions of it and larger than it
+@pytest.mark.parametrize("w,h,cw,ch", [(1, 1, 1, 1), (31, 7, 13, 3), (32, 8, 32, 8), (33, 9, 11, 9),
+                                       (97, 61, 32, 21), (40, 17, 81, 35)])
+@pytest.mark.parametrize("fmt", ["fp32", "fp16"])
+def test_composite_tile_edges(api, oracle, w, h, cw, ch, fmt):
+    rng = np.random.default_rng(w * h + cw)
+    cloud, bg = I.synthetic_frame(rng, ch, cw), rng.uniform(0.0, 2.0, (h, w, 4)).astype(np.float32)
+    cloud = cloud.astype(np.float16) if fmt == "fp16" else cloud
+    got = api.composite(_t(cloud), _t(bg)).cpu().numpy()
+    assert np.abs(got - oracle.composite(cloud.astype(np.float64), bg)).max() <= 2e-6
