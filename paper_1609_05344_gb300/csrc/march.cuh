@@ -507,8 +507,11 @@ __device__ __forceinline__ unsigned march_tile(
     bool alive = false;
     const float xf = (float)x, yf = (float)y;
     if (inside) {
-        // quick FP32 test for rays that cannot reach the layer (a 1e-4 margin
-        // keeps every undecided ray on the exact path below)
+        // quick FP32 test for rays that cannot reach the layer.  It takes the 10-bit
+        // high halves of the slopes only, so its d_z is off by up to 2^-10 of the
+        // image plane's extent, more than the thresholds' 1e-4 margin: a ray that
+        // grazes the layer near the far clip can be dropped (up to 37 pixels of a
+        // 957x541 image, up to 0.1 in RGBA).
         const float qx = fmaf(yf, v.vyh[0], fmaf(xf, v.vxh[0], v.v00h[0]));
         const float qy = fmaf(yf, v.vyh[1], fmaf(xf, v.vxh[1], v.v00h[1]));
         const float qz = fmaf(yf, v.vyh[2], fmaf(xf, v.vxh[2], v.v00h[2]));
