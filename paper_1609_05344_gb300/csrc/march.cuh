@@ -14,6 +14,12 @@
 // integer adds, no rounding.  The texel index is the top log2(N) bits, the
 // interpolation weight the next 23 bits.  Radiance and the optical-depth sum
 // are FP32.
+//
+// Times in the comments below compare a choice with its alternatives in one run of
+// its time; cameras and builds differ from comment to comment (1920x1080 x 8 steps of
+// the standard FP32 volume: 83 to 116 us), so figures of different comments do not
+// compare.  Now: 116 us for the mean of a 32-frame orbit with the L2 flushed, 94 us a
+// pass with inputs in turn.
 #pragma once
 
 #include "common.cuh"

@@ -186,7 +186,8 @@ int build_view(const cloud_volume *vol, const cloud_params *prm, const cloud_cam
 
 // ---------------------------------------------------------------------------
 // Launch-configuration selection per (storage precision, six light steps or another
-// number): what the autotuner found fastest or the caller set, -1 for the default.  A
+// number), the key of cloud_set_launch_config, which volumes of every kind share: what
+// the autotuner found fastest or the caller set, -1 for the default.  A
 // single view too small to fill the GPU has a choice of its own: -1 leaves it to
 // small_shape below, which the eight configurations hardly ever beat there.
 namespace {
